@@ -13,8 +13,15 @@
 //       of a warp walk units of the same length and stay in step (a block-wide exclusive
 //       scan over per-warp bucket counters is the work distributor);
 //   (3) walks each unit's rows: per row the four face bounds, the tightest upper and
-//       lower bound certified once each (the filter's bracket of Section 4's orientation
-//       values, see tet_math.cuh), and the interval ORed into the grid's words.
+//       lower bound certified once each (the filter of Section 4's orientation values,
+//       voxtet_rows.cuh), and the interval ORed into the grid's words.
+// What bounds it: instruction issue, the L1 data path (record loads of random slots, the
+// ORs) and, on finer grids, the rate at which an SM can send ORs to L2.  Measured on GB300
+// with timing-only copies, 1.3 M-tet sliver mesh at 512^3 (258 us): load, classification and
+// face data 58 us, the slices' row ranges 29, the sort 14, the units' record loads 28, the
+// rows' bounds 61, the ORs 68.  Biased bounds (no separate bracket), one add-and-round per
+// side, 16-word records and the rows' range from four lines took the kernel from 274 to 257 us
+// there and from 1027 to 1002 us at 1024^3 (212 M warp instructions against 221 M).
 // Tets this kernel does not take -- zero volume (skipped), wider than 2^20 lattice
 // units or use_filter = 0 (exact kernel), or more than kSuSlices slices or kSuRows rows
 // per slice (listed at the back of the tet queue for the span kernel) -- are counted or
@@ -27,6 +34,7 @@
 #include "voxtet.h"
 #include "tet_math.cuh"
 #include "voxtet_device.cuh"
+#include "voxtet_rows.cuh"
 #include "voxtet_slices.cuh"
 
 namespace voxtet {
@@ -34,19 +42,18 @@ namespace voxtet {
 constexpr int kSuWarps = kSuBlock / 32;
 constexpr int kSuBuckets = 64;                           // row counts 1..63 one bucket each, >= 64 together
 constexpr int kSuCounters = kSuBuckets * kSuWarps;       // bucket-major, one counter per warp of each bucket
-constexpr int kSuRec = 28;  // floats per tet record: 24 used; 7 groups of 16 bytes, an odd number,
+constexpr int kSuRec = 20;  // floats per tet record: 16 used; 5 groups of 16 bytes, an odd number,
                             // so that lanes loading records of random slots spread over all banks
 constexpr int kSuStage = 64;                             // staged uncertain rows per block (about 5 per tile)
 constexpr uint32_t kSuEmpty = 0xFFFFFFFFu;               // a slice without candidate rows
 static_assert(kSuBlock == 128 && kSuSlices <= 32 && kSuRows == 1024, "unit fields: 7 + 5 bits; rows in 10 bits");
 
-// Tet record (kSuRec floats per slot).  The faces bounding a from above (Dx < 0) fill slots
-// U0..U2 and those bounding it from below (Dx > 0) slots L0..L2, unused slots a neutral face
-// (alpha = +inf, beta = gamma = 0: its bound is +inf and never the smallest).  Each U/L pair
-// is adjacent.  Fields: alpha U0 L0 U1 L1 U2 L2 | beta (same order) | gamma (same order) |
-// bracket of the upper side, of the lower side | na - 1 | i0 (int bits) | 64-bit grid word
-// offset of the box's row (b, c) = (0, 0).
-constexpr int kRecAl = 0, kRecBe = 6, kRecGa = 12, kRecDU = 18, kRecDL = 19, kRecHi = 20, kRecI0 = 21, kRecBase = 22;
+// Tet record (kSuRec words per slot): alpha' of the four faces | beta | gamma | E of the upper
+// and of the lower side, i0 | (na - 1) << 16 | upper slots << 30, j0 | (l0 - z0) << 16.  Upper faces fill the slots from the
+// front and lower faces from the back; a face parallel to x leaves a neutral upper slot (alpha' =
+// +infinity) between them.  Slot 0 is always an upper face and slot 3 a lower one.
+constexpr int kRecB = 4, kRecG = 8, kRecEU = 12, kRecEL = 13, kRecX = 14, kRecYZ = 15;
+constexpr int kSuColumns = 1 << 14;  // most samples along x of a tet's box (14 bits hold na - 1)
 
 // Shared memory of one block (dynamic), for tets of at most SL slices.
 template <int SL>
@@ -54,10 +61,10 @@ struct SuSmem {
   float rec[kSuBlock * kSuRec];
   // per tet slot, slice k of its tet: b_lo | (n - 1) << 10, or kSuEmpty
   uint32_t slice[SL][kSuBlock];
-  // the tile's units sorted by row count, longest first: slot | k << 7
-  uint16_t unit[kSuBlock * SL];
-  uint32_t hist[kSuCounters];
-  uint32_t cur[kSuCounters + 1];
+  // the tile's units sorted by row count, longest first: slot | k << 7 | b_lo << 12 | (n - 1) << 22
+  uint32_t unit[kSuBlock * SL];
+  uint32_t hist[kSuCounters];  // unit counts, then (after the scan) cursors
+  uint32_t total;
   uint32_t warp_tot[kSuWarps];
   RowStageN<kSuStage> stage;
   long long tile;
@@ -65,54 +72,11 @@ struct SuSmem {
 
 // 16-slice tiles fit 7 blocks per SM (228 KB, 1 KB reserved per block), 32-slice tiles 5
 static_assert(sizeof(SuSmem<kSuSlicesSmall>) <= 31 * 1024, "slice-unit kernel shared memory: seven blocks per SM");
-static_assert(sizeof(SuSmem<kSuSlices>) <= 44 * 1024, "slice-unit kernel shared memory: five blocks per SM");
+static_assert(sizeof(SuSmem<kSuSlices>) <= 44 * 1024 + 512, "slice-unit kernel shared memory: five blocks per SM");
 
 // Counter of a unit with n rows emitted by warp w: longer units first.
 __device__ __forceinline__ int su_counter(int n, int w) {
   return (kSuBuckets - min(n, kSuBuckets)) * kSuWarps + w;
-}
-
-// Edges of a tet for the per-slice row range, its vertices sorted by z (z0 <= z1 <= z2 <=
-// z3): edge e = (p, q) meets the plane at height Z at y = yp + (Z - zp) k, k = (yq - yp) /
-// (zq - zp) (0 for a horizontal edge, whose end points other edges reach).  Z - zp and the
-// integer differences are exact in float; k comes from __fdividef (at most 2 ulp off for
-// divisors in [1, 2^22]), so a crossing point is within 4u 2^22 + u 2^22 = 1.25 lattice
-// units of the true one, inside the 2 units the range is widened by.
-// Order: 01 02 03 12 13 23.  Slices below z1 cross 01 02 03, slices in [z1, z2] cross
-// 02 03 12 13, above z2 03 13 23.  A horizontal edge (k = 0) yields only its first end
-// point, so in [z1, z2] vertex 2 is added at Z = z2 (02 and 12 are both horizontal when
-// z0 = z1 = z2, and 23, which starts there, belongs to the slices above); vertex 1 always
-// comes from 12 and 13, which start at it.
-struct SuEdges {
-  float zp[6], yp[6], k[6];
-  int z1, z2;
-};
-
-__device__ __forceinline__ void su_edges(const int3 V[4], SuEdges &E) {
-  int z[4] = {V[0].z, V[1].z, V[2].z, V[3].z};
-  int y[4] = {V[0].y, V[1].y, V[2].y, V[3].y};
-#define VOXTET_CSWAP(a, b)                                  \
-  if (z[b] < z[a]) {                                        \
-    const int tz = z[a], ty = y[a];                         \
-    z[a] = z[b]; y[a] = y[b]; z[b] = tz; y[b] = ty;         \
-  }
-  VOXTET_CSWAP(0, 1)
-  VOXTET_CSWAP(2, 3)
-  VOXTET_CSWAP(0, 2)
-  VOXTET_CSWAP(1, 3)
-  VOXTET_CSWAP(1, 2)
-#undef VOXTET_CSWAP
-#pragma unroll
-  for (int e = 0; e < 6; ++e) {
-    const int pi = e < 3 ? 0 : (e < 5 ? 1 : 2);
-    const int qi = e < 3 ? e + 1 : (e < 5 ? e - 1 : 3);
-    const int dz = z[qi] - z[pi];
-    E.zp[e] = (float)z[pi];
-    E.yp[e] = (float)y[pi];
-    E.k[e] = dz != 0 ? __fdividef((float)(y[qi] - y[pi]), (float)dz) : 0.f;
-  }
-  E.z1 = z[1];
-  E.z2 = z[2];
 }
 
 // Phase (1) for tet t of this thread (t < 0: none).  Returns the slices whose entries it
@@ -156,7 +120,7 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, SuSmem<SL>
     p.tetq[k] = (uint32_t)t;
     return 0;
   }
-  if (bx.nc > SL || bx.nb > kSuRows) {  // the span kernel takes it (list mode)
+  if (bx.nc > SL || bx.nb > kSuRows || bx.na > kSuColumns) {  // the span kernel takes it (list mode)
     const unsigned k = atomicAdd(&p.hdr->listq_count, 1u);
     p.tetq[p.n_tets - 1 - k] = (uint32_t)t;
     return 0;
@@ -193,23 +157,24 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, SuSmem<SL>
   // and one with Dx > 0 (the four gradients sum to zero, at most two vanish).
   float *rec = sm.rec + tid * kSuRec;
   const float fb = (float)(bx.nb - 1), fc = (float)(bx.nc - 1);
-  float dU = 0.f, dL = 0.f;
-  int cu = 0, cl = 0;
+  float eU = 0.f, eL = 0.f;
+  int cu = 0, cl = 3;
   i64 zL0 = 0, zDy0 = 0, zDz0 = 0, zL1 = 0, zDy1 = 0, zDz1 = 0;
   int nz = 0;
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
-    const i64 Dx = Nx[m] << p.sh, Dy = Ny[m] << p.sh, Dz = Nz[m] << p.sh;
-    if (Dx != 0) {
-      float a, b, g, d;
-      filter_slot(L[m], Dx, Dy, Dz, fb, fc, a, b, g, d);
-      const int o = Dx < 0 ? 2 * cu++ : 2 * cl++ + 1;
-      rec[kRecAl + o] = a;
-      rec[kRecBe + o] = b;
-      rec[kRecGa + o] = g;
-      if (Dx < 0) dU = fmaxf(dU, d);
-      else dL = fmaxf(dL, d);
+    if (Nx[m] != 0) {
+      float a, b, g;
+      const float e = face_bound<STRICT>(L[m], Nx[m], Ny[m], Nz[m], p.sh, fb, fc, a, b, g);
+      const bool up = Nx[m] < 0;
+      const int o = up ? cu++ : cl--;
+      if (up) eU = fmaxf(eU, e);
+      else eL = fmaxf(eL, e);
+      rec[o] = a;
+      rec[kRecB + o] = b;
+      rec[kRecG + o] = g;
     } else {
+      const i64 Dy = Ny[m] << p.sh, Dz = Nz[m] << p.sh;
       if (nz == 0) {
         zL0 = L[m]; zDy0 = Dy; zDz0 = Dz;
       } else {
@@ -218,74 +183,46 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, SuSmem<SL>
       ++nz;
     }
   }
-  const float INF = __int_as_float(0x7f800000);
-  for (int q = cu; q < 3; ++q) {
-    rec[kRecAl + 2 * q] = INF;
-    rec[kRecBe + 2 * q] = 0.f;
-    rec[kRecGa + 2 * q] = 0.f;
+  for (; cu <= cl; ++cu) {
+    rec[cu] = __int_as_float(0x7f800000);
+    rec[kRecB + cu] = 0.f;
+    rec[kRecG + cu] = 0.f;
   }
-  for (int q = cl; q < 3; ++q) {
-    rec[kRecAl + 2 * q + 1] = INF;
-    rec[kRecBe + 2 * q + 1] = 0.f;
-    rec[kRecGa + 2 * q + 1] = 0.f;
-  }
-  rec[kRecDU] = dU;
-  rec[kRecDL] = dL;
-  rec[kRecHi] = (float)(bx.na - 1);
-  rec[kRecI0] = __int_as_float(bx.i0);
-  *reinterpret_cast<long long *>(rec + kRecBase) = ((long long)(bx.l0 - p.z0) * p.ry + bx.j0) * p.W;
+  rec[kRecEU] = eU;
+  rec[kRecEL] = eL;
+  rec[kRecX] = __uint_as_float((uint32_t)bx.i0 | ((uint32_t)(bx.na - 1) << 16) | ((uint32_t)cu << 30));
+  rec[kRecYZ] = __uint_as_float((uint32_t)bx.j0 | ((uint32_t)(bx.l0 - p.z0) << 16));
   // Candidate rows of each slice: the cross-section's y-extent (a superset of the rows with
   // samples), narrowed exactly by the faces parallel to x.  Each unit is counted (no rank is
   // needed here, so the count does not wait on the shared-memory atomic).
-  SuEdges EG;
-  int kA = bx.nc, kB = bx.nc;
+  RowRange R;
   if (CULL) {
-    su_edges(V, EG);
-    // slices k < kA lie below z1, k < kB at or below z2
-    kA = min(max(((EG.z1 - s + (1 << p.sh) - 1) >> p.sh) - bx.l0, 0), bx.nc);
-    kB = min(max(((EG.z2 - s) >> p.sh) + 1 - bx.l0, kA), bx.nc);
+    row_range(V, bx, p.sh, R);
+  } else {
+    R.kL0 = R.kL1 = R.kU0 = R.kU1 = 0.f;
+    R.aL0 = R.aL1 = 0.f;
+    R.aU0 = R.aU1 = fb;
   }
   int units = 0;
-  // one slice: its rows narrowed by the x-parallel faces, counted, recorded
-  auto emit = [&](int k, int b_lo, int b_hi) {
-    if (nz > 0) narrow_by_row_constraint<STRICT>(zL0 + zDz0 * (i64)k, zDy0, b_lo, b_hi);
-    if (nz > 1) narrow_by_row_constraint<STRICT>(zL1 + zDz1 * (i64)k, zDy1, b_lo, b_hi);
-    uint32_t e = kSuEmpty;
-    if (b_hi >= b_lo) {
-      const int n = b_hi - b_lo + 1;
-      atomicAdd(&sm.hist[su_counter(n, warp)], 1u);
-      e = (uint32_t)b_lo | ((uint32_t)(n - 1) << 10);
+  float cf = 0.f;
+  for (int k = 0; k < bx.nc; ++k, cf += 1.f) {
+    float flo, fhi;
+    slice_range(R, cf, fb, flo, fhi);
+    bool any = flo <= fhi;
+    uint32_t b_lo = __float_as_uint(flo) - kMagicBits, n1 = __float_as_uint(fhi) - __float_as_uint(flo);
+    if (nz > 0 && any) {
+      int lo = (int)b_lo, hi = (int)(b_lo + n1);
+      narrow_by_row_constraint<STRICT>(zL0 + zDz0 * (i64)k, zDy0, lo, hi);
+      if (nz > 1) narrow_by_row_constraint<STRICT>(zL1 + zDz1 * (i64)k, zDy1, lo, hi);
+      any = lo <= hi;
+      b_lo = (uint32_t)lo;
+      n1 = (uint32_t)(hi - lo);
+    }
+    if (any) {
+      atomicAdd(&sm.hist[su_counter((int)n1 + 1, warp)], 1u);
       ++units;
     }
-    sm.slice[k][tid] = e;
-  };
-  if (CULL) {
-    const int step = 1 << p.sh;
-    int Z = s + (bx.l0 << p.sh);
-    // the edges' first end points are vertices 0 (01 02 03), 1 (12 13) and 2 (23)
-    const float zs0 = EG.zp[0], zs1 = EG.zp[3], zs2 = EG.zp[5], ys0 = EG.yp[0], ys1 = EG.yp[3], ys2 = EG.yp[5];
-    const float k0 = EG.k[0], k1 = EG.k[1], k2 = EG.k[2], k3 = EG.k[3], k4 = EG.k[4], k5 = EG.k[5];
-    for (int k = 0; k < bx.nc; ++k, Z += step) {
-      // the slice's crossing points, edges chosen by selects (one straight-line body for all
-      // slices): below z1 03 01 02; in [z1, z2] 03 02 12 13 and vertex 2 at z2; above 03 13 23
-      const float Zf = (float)Z;
-      const bool pa = k < kA, pb = !pa && k < kB, pc = !pa && !pb;
-      const float d0 = Zf - zs0, d1 = Zf - zs1, d2 = Zf - zs2;
-      const float y1 = __fmaf_rn(d0, k2, ys0);
-      const float y2 = __fmaf_rn(pc ? d1 : d0, pa ? k0 : (pb ? k1 : k4), pc ? ys1 : ys0);
-      const float y3 = __fmaf_rn(pa ? d0 : (pb ? d1 : d2), pa ? k1 : (pb ? k3 : k5), pa ? ys0 : (pb ? ys1 : ys2));
-      const float y4 = pb ? __fmaf_rn(d1, k4, ys1) : y1;
-      const float y5 = pb && Z == EG.z2 ? ys2 : y1;
-      const float ymin = fminf(fminf(fminf(y1, y2), fminf(y3, y4)), y5);
-      const float ymax = fmaxf(fmaxf(fmaxf(y1, y2), fmaxf(y3, y4)), y5);
-      // the y-extent widened by 2 lattice units, in rows
-      const int ylo = (int)floorf(ymin) - 2, yhi = (int)ceilf(ymax) + 2;
-      const int b_lo = max(((ylo + s - 1) >> p.sh) - bx.j0, 0);
-      const int b_hi = min(((yhi - s) >> p.sh) - bx.j0, bx.nb - 1);
-      emit(k, b_lo, b_hi);
-    }
-  } else {
-    for (int k = 0; k < bx.nc; ++k) emit(k, 0, bx.nb - 1);
+    sm.slice[k][tid] = any ? b_lo | (n1 << 10) : kSuEmpty;
   }
   return units ? bx.nc : 0;
 }
@@ -315,88 +252,54 @@ __device__ __forceinline__ uint32_t su_block_scan(SuSmem<SL> &sm, uint32_t v, ui
   return before;
 }
 
-// Filter data of one unit (a slice of one tet) for its rows.
-struct SuUnit {
-  float aU0, aL0, aU1, aL1, aU2, aL2;  // alpha + gamma c of each face slot
-  float bU0, bL0, bU1, bL1, bU2, bL2;  // beta of each face slot
-  float dU, dL, fhi0;
-  int i0;
-};
-
-// One row at bf (the row index as a float): its interval, ORed into `row`.  Returns true if
-// the filter could not certify the row (nothing is written then; the caller queues it).
-template <bool STRICT, bool CLAMP>
-__device__ __forceinline__ bool su_row(const SuUnit &u, float bf, uint32_t *row) {
-  // tightest bound of each side; the bracket of the smallest of the faces' values is the
-  // smallest of their brackets, so one certification per side suffices
-  const float TU = fminf(__fmaf_rn(u.bU0, bf, u.aU0), fminf(__fmaf_rn(u.bU1, bf, u.aU1), __fmaf_rn(u.bU2, bf, u.aU2)));
-  const float TL = fminf(__fmaf_rn(u.bL0, bf, u.aL0), fminf(__fmaf_rn(u.bL1, bf, u.aL1), __fmaf_rn(u.bL2, bf, u.aL2)));
-  float thU = __fadd_ru(TU, u.dU), tlU = __fsub_rd(TU, u.dU);
-  float thL = __fadd_ru(TL, u.dL), tlL = __fsub_rd(TL, u.dL);
-  if (CLAMP) {  // only where the bound can change the row (as in the span kernel)
-    tlU = fmaxf(tlU, STRICT ? 0.f : -1.f);
-    thU = fminf(thU, STRICT ? u.fhi0 + 1.f : u.fhi0);
-    tlL = fmaxf(tlL, STRICT ? -u.fhi0 : -u.fhi0 - 1.f);
-    thL = fminf(thL, STRICT ? 1.f : 0.f);
-  }
-  float lo, hi;
-  bool amb;
-  if (STRICT) {  // a < T: a <= ceil(T) - 1; a > -T: a >= 1 - ceil(T)
-    const float cU = ceilf(tlU), cL = ceilf(tlL);
-    amb = (cU < thU) | (cL < thL);
-    hi = fminf(u.fhi0, cU - 1.f);
-    lo = fmaxf(0.f, 1.f - cL);
-  } else {  // a <= T: a <= floor(T); a >= -T: a >= -floor(T)
-    const float fU = floorf(thU), fL = floorf(thL);
-    amb = (fU > tlU) | (fL > tlL);
-    hi = fminf(u.fhi0, fU);
-    lo = fmaxf(0.f, -fL);
-  }
-  const bool live = !amb && lo <= hi;
-  // lo, hi are integral floats in [0, na - 1] when live; otherwise every access below is
-  // predicated off
-  const int x0 = u.i0 + small_float_to_int(lo);
-  const int x1 = u.i0 + small_float_to_int(hi);
-  or_span_lanes(row, x0, x1, live);
-  return amb;
-}
-
 // Phase (3): rows b0 .. b0 + n - 1 of slice k of the tet in `slot` (tet index t).
 template <bool STRICT, bool CLAMP, int SL>
 __device__ __forceinline__ void su_walk(const Params &p, SuSmem<SL> &sm, int slot, long long t, int k, int b0, int n) {
   const float4 *R = reinterpret_cast<const float4 *>(sm.rec + slot * kSuRec);
-  const float4 q0 = R[0], q1 = R[1], q2 = R[2], q3 = R[3], q4 = R[4], q5 = R[5];
-  const float cf = (float)k;
-  SuUnit u;
-  u.aU0 = __fmaf_rn(q3.x, cf, q0.x);
-  u.aL0 = __fmaf_rn(q3.y, cf, q0.y);
-  u.aU1 = __fmaf_rn(q3.z, cf, q0.z);
-  u.aL1 = __fmaf_rn(q3.w, cf, q0.w);
-  u.aU2 = __fmaf_rn(q4.x, cf, q1.x);
-  u.aL2 = __fmaf_rn(q4.y, cf, q1.y);
-  u.bU0 = q1.z; u.bL0 = q1.w; u.bU1 = q2.x; u.bL1 = q2.y; u.bU2 = q2.z; u.bL2 = q2.w;
-  u.dU = q4.z;
-  u.dL = q4.w;
-  u.fhi0 = q5.x;
-  u.i0 = __float_as_int(q5.y);
-  const long long base = (long long)(((unsigned long long)__float_as_uint(q5.w) << 32) | __float_as_uint(q5.z));
-  const long long W = p.W;
-  uint32_t *row = p.out + base + (long long)k * p.ry * W + (long long)b0 * W;
+  const float4 qa = R[0], qb = R[1], qg = R[2], qi = R[3];
+  const float cf = (float)k, INF = __int_as_float(0x7f800000);
+  const uint32_t xx = __float_as_uint(qi.z), yz = __float_as_uint(qi.w);
+  const uint32_t nup = xx >> 30;
+  const bool up1 = nup >= 2, up2 = nup >= 3;
+  const float a1 = __fmaf_rn(qg.y, cf, qa.y), a2 = __fmaf_rn(qg.z, cf, qa.z);
+  RowFaces f;
+  f.aU0 = __fmaf_rn(qg.x, cf, qa.x);
+  f.bU0 = qb.x;
+  f.aU1 = up1 ? a1 : INF;
+  f.bU1 = up1 ? qb.y : 0.f;
+  f.aU2 = up2 ? a2 : INF;
+  f.bU2 = up2 ? qb.z : 0.f;
+  f.aL0 = __fmaf_rn(qg.w, cf, qa.w);
+  f.bL0 = qb.w;
+  f.aL1 = up1 ? -INF : a1;
+  f.bL1 = up1 ? 0.f : qb.y;
+  f.aL2 = up2 ? -INF : a2;
+  f.bL2 = up2 ? 0.f : qb.z;
+  f.eU = qi.x;
+  f.eL = qi.y;
+  row_magic<STRICT>(f, (int)(xx & 0xFFFFu), (int)((xx >> 16) & 0x3FFFu));
+  // rows of the slab from its first: below 2^32 for every accepted grid
+  const uint32_t r0 = ((yz >> 16) + (uint32_t)k) * (uint32_t)p.ry + (yz & 0xFFFFu) + (uint32_t)b0;
+  uint32_t *const row = p.out + (size_t)r0 * (uint32_t)p.W - kMagicWord;
+  uint32_t off = 0;
   float bf = (float)b0;
   // uncertain rows are collected as bits, 32 rows at a time, and queued after the rows, so
   // that the row loop has no call in it
-  for (int r0 = 0; r0 < n; r0 += 32) {
-    const int r1 = min(n, r0 + 32);
+  for (int s0 = 0; s0 < n; s0 += 32) {
+    const int s1 = min(n, s0 + 32);
     uint32_t amb = 0;
-    for (int r = r0; r < r1; ++r) {
-      amb |= (uint32_t)su_row<STRICT, CLAMP>(u, bf, row) << (r - r0);
+    for (int r = s0; r < s1; ++r) {
+      uint32_t lo, hi;
+      bool live;
+      amb |= (uint32_t)row_bounds<STRICT, CLAMP>(f, bf, lo, hi, live) << (r - s0);
+      row_or(row, off, lo, hi, live);
       bf += 1.f;
-      row += W;
+      off += (uint32_t)p.W;
     }
     while (amb) {
       const int j = __ffs(amb) - 1;
       amb &= amb - 1u;
-      queue_row_staged(p, sm.stage, t, b0 + r0 + j, k);
+      queue_row_staged(p, sm.stage, t, b0 + s0 + j, k);
     }
   }
 }
@@ -435,30 +338,29 @@ __global__ void __launch_bounds__(kSuBlock, SL == kSuSlicesSmall ? 7 : 5) k_slic
       const uint32_t c0 = sm.hist[2 * tid], c1 = sm.hist[2 * tid + 1];
       uint32_t all = 0;
       const uint32_t before = su_block_scan(sm, c0 + c1, all);
-      sm.cur[2 * tid] = before;
-      sm.cur[2 * tid + 1] = before + c0;
-      if (tid == kSuBlock - 1) sm.cur[kSuCounters] = all;
-      sm.hist[2 * tid] = 0u;  // ready for the next tile (read no more in this one)
-      sm.hist[2 * tid + 1] = 0u;
+      sm.hist[2 * tid] = before;
+      sm.hist[2 * tid + 1] = before + c0;
+      if (tid == 0) sm.total = all;
       __syncthreads();
     }
-    const uint32_t total = sm.cur[kSuCounters];
+    const uint32_t total = sm.total;
 #pragma unroll 4
     for (int k = 0; k < nc; ++k) {
       const uint32_t e = sm.slice[k][tid];
       if (e == kSuEmpty) continue;
       const int n = (int)(e >> 10) + 1;
-      const uint32_t pos = atomicAdd(&sm.cur[su_counter(n, tid >> 5)], 1u);
-      sm.unit[pos] = (uint16_t)(tid | (k << 7));
+      const uint32_t pos = atomicAdd(&sm.hist[su_counter(n, tid >> 5)], 1u);
+      sm.unit[pos] = (uint32_t)tid | ((uint32_t)k << 7) | (e << 12);
     }
     __syncthreads();
     if (tid == 0) ctr.spans += total;
+    sm.hist[2 * tid] = 0u;  // ready for the next tile's counts (a barrier comes before them)
+    sm.hist[2 * tid + 1] = 0u;
     // (3) walk the units, longest first; a warp takes 32 neighbouring units of the order
     for (uint32_t i = tid; i < total; i += kSuBlock) {
       const uint32_t u = sm.unit[i];
-      const int slot = (int)(u & 127u), k = (int)(u >> 7);
-      const uint32_t e = sm.slice[k][slot];
-      const int b0 = (int)(e & 1023u), n = (int)(e >> 10) + 1;
+      const int slot = (int)(u & 127u), k = (int)((u >> 7) & 31u);
+      const int b0 = (int)((u >> 12) & 1023u), n = (int)(u >> 22) + 1;
       const long long tt = STRIDED ? base + (long long)slot * p.tile_stride : base + slot;
       ctr.rows += (unsigned)n;
       su_walk<STRICT, CLAMP, SL>(p, sm, slot, tt, k, b0, n);
