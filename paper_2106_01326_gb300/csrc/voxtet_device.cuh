@@ -43,13 +43,13 @@ struct Header {
   int status_bits;
   unsigned tetq_count;  // tets queued for the exact kernel
   unsigned rowq_count;  // rows queued for the exact kernel (may exceed the capacity)
-  unsigned listq_count;  // tets the slice-unit kernel left to the span kernel (kept at the back of tetq)
+  unsigned listq_count;  // tets of a thin slab, kept at the back of tetq (k_slab_list)
   unsigned long long tile_counter;
   unsigned long long spans;
   unsigned long long rows;
   unsigned long long degenerate;
   unsigned long long wide;
-  unsigned long long list_tile_counter;  // tiles claimed by the span kernel in list mode
+  unsigned long long list_rows;  // rows of their boxes, over all slices
   unsigned long long reserved[24];
 };
 static_assert(sizeof(Header) == 256, "header is 256 bytes");
@@ -67,7 +67,7 @@ struct Params {
   long long n_verts;
   uint32_t *out;
   Header *hdr;
-  uint32_t *tetq;   // [n_tets]
+  uint32_t *tetq;   // [n_tets]; a thin slab's tets are listed from the back, the queue fills from the front
   RowItem *rowq;    // [q_cap]
   uint32_t *redo;   // [ceil(n_tets / 32)] bitmap
   unsigned q_cap;
@@ -78,10 +78,9 @@ struct Params {
   int span_rows;    // target bounding-box rows per span
   int exact_all;    // 1: every tet goes to the exact kernel
   int max_slices;   // slices a span may hold (16 or 32): the slice table's rows in dynamic shared memory
-  int cull;         // 1: skip rows outside each slice's cross-section (batched kernel)
   long long big_tiles;  // single-mesh launch: tiles of kTile tets before the kSmallTile tail
   long long tile_stride;  // > 0: tile k holds tets k + j * tile_stride (slab launches), else contiguous tiles
-  int list_mode;    // span kernel: 1 = its tets are the hdr->listq_count ones listed at the back of tetq
+  int lg;           // slice-unit kernel: log2 of the threads that share a tet
   int vflags;       // exact kernel: 1 = fold the vertices' error bits (verts4[i].w) into the status
 };
 
@@ -117,6 +116,15 @@ static cudaError_t launch_chained(void (*kernel)(Args...), unsigned grid, unsign
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Actual &&>(args)...);
+}
+
+// *p |= bits for a pointer that the compiler does not know to point to device memory: the batched
+// kernels read theirs from a job's Params in shared memory, and atomicOr is then a generic atomic,
+// held up like one that returns its value (measured on GB300, 64 meshes of 1k-1M tets on 64^3-512^3
+// grids: 1.52 ms with atomicOr, 0.87 with this; where the pointer is a kernel's own parameter
+// atomicOr is the faster one, 263 against 271 us for the sliver mesh at 512^3).
+__device__ __forceinline__ void red_or(uint32_t *p, uint32_t bits) {
+  asm volatile("red.relaxed.gpu.global.or.b32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "r"(bits));
 }
 
 // ------------------------------------------------------------------ OR writes
@@ -157,9 +165,8 @@ __device__ __forceinline__ void or_span_lanes(uint32_t *__restrict__ row, int x0
 // (already recorded by the snap kernel).
 __device__ __forceinline__ bool load_tet(const Params &p, long long t, int3 V[4], int &err) {
   const int4 q = p.tets[t];
-  const unsigned long long nv = (unsigned long long)p.n_verts;
-  if (q.x < 0 || q.y < 0 || q.z < 0 || q.w < 0 || (unsigned long long)q.x >= nv || (unsigned long long)q.y >= nv ||
-      (unsigned long long)q.z >= nv || (unsigned long long)q.w >= nv) {
+  const unsigned nv = (unsigned)p.n_verts;  // below 2^31, so a negative index compares above it
+  if ((unsigned)q.x >= nv || (unsigned)q.y >= nv || (unsigned)q.z >= nv || (unsigned)q.w >= nv) {
     err |= kErrIndex;
     return false;
   }
@@ -234,7 +241,12 @@ __device__ __forceinline__ void slice_rows_sorted(const EdgeLines &E, int Z, int
 // Queue row (b, c) of tet t for the exact kernel; if the row queue is full, flag the
 // whole tet for an exact redo instead.
 __device__ __forceinline__ void queue_row(const Params &p, long long t, int b, int c) {
-  const unsigned k = atomicAdd(&p.hdr->rowq_count, 1u);
+  // one atomic for the lanes that are here together
+  const unsigned m = __activemask(), lane = threadIdx.x & 31;
+  const int first = __ffs(m) - 1;
+  unsigned k = 0;
+  if ((int)lane == first) k = atomicAdd(&p.hdr->rowq_count, (unsigned)__popc(m));
+  k = __shfl_sync(m, k, first) + (unsigned)__popc(m & ((1u << lane) - 1u));
   if (k < p.q_cap) {
     RowItem it;
     it.tet = (uint32_t)t;
@@ -334,8 +346,9 @@ struct TileCounters {
 };
 
 
-// Adds a block's counters to a mesh's header: one atomic per warp and counter.
-__device__ __forceinline__ void flush_counters(Header *hdr, TileCounters &ctr) {
+// Adds a block's counters to a mesh's header: one atomic per warp and counter.  Error bits also
+// go to `status` if one is given (a batch job's status word).
+__device__ __forceinline__ void flush_counters(Header *hdr, TileCounters &ctr, int *status = nullptr) {
   const int lane = threadIdx.x & 31;
   unsigned long long rows_w = ctr.rows, deg_w = ctr.degenerate, wide_w = ctr.wide;
 #pragma unroll
@@ -350,6 +363,7 @@ __device__ __forceinline__ void flush_counters(Header *hdr, TileCounters &ctr) {
     if (deg_w) atomicAdd(&hdr->degenerate, deg_w);
     if (wide_w) atomicAdd(&hdr->wide, wide_w);
     if (err) atomicOr(&hdr->status_bits, err);
+    if (err && status) atomicOr(status, err);
   }
   if (threadIdx.x == 0 && ctr.spans) atomicAdd(&hdr->spans, ctr.spans);
   ctr = TileCounters();

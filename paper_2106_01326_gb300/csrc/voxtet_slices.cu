@@ -15,21 +15,23 @@
 //   (3) walks each unit's rows: per row the four face bounds, the tightest upper and
 //       lower bound certified once each (the filter of Section 4's orientation values,
 //       voxtet_rows.cuh), and the interval ORed into the grid's words.
-// What bounds it: instruction issue, the L1 data path (record loads of random slots, the
-// ORs) and, on finer grids, the rate at which an SM can send ORs to L2.  Measured on GB300
-// with timing-only copies, 1.3 M-tet sliver mesh at 512^3 (258 us): load, classification and
-// face data 58 us, the slices' row ranges 29, the sort 14, the units' record loads 28, the
-// rows' bounds 61, the ORs 68.  Biased bounds (no separate bracket), one add-and-round per
-// side, 16-word records and the rows' range from four lines took the kernel from 274 to 257 us
-// there and from 1027 to 1002 us at 1024^3 (212 M warp instructions against 221 M).
-// Tets this kernel does not take -- zero volume (skipped), wider than 2^20 lattice
-// units or use_filter = 0 (exact kernel), or more than kSuSlices slices or kSuRows rows
-// per slice (listed at the back of the tet queue for the span kernel) -- are counted or
-// queued exactly as the span kernel would.  Rows the filter cannot certify go to the
-// same row queue, solved afterwards by the exact kernel.
+// Where a mesh has too few tets for a thread each to fill the chip, or tets of more slices than a
+// thread takes, a group of 2^lg threads shares a tet and its slices (su_group_log2); slices or rows
+// past that are taken in further windows of the same tile.  A batch's jobs run in one launch
+// (k_slices_batched), a thin slab's tets from a list (LIST).
+// What bounds it: instruction issue and, on finer grids, the rate at which ORs reach L2, half of
+// them across the dies.  Measured on GB300 with timing-only copies, 1.3 M-tet sliver mesh: at
+// 512^3 261 us a call, of these 65 for the ORs, 100 for the rest of the rows, 45 for the slices'
+// row ranges and the sort, 40 for load, classification and face data; at 1024^3 1020 us, 505 for
+// the ORs (213 M of them) and 360 for the rest of the rows.  ORing a tile's rows in shared memory
+// first and the words once into the grid took 9 times fewer ORs but a sixth more instructions
+// (302 and 1100 us).
+// Tets wider than 2^20 lattice units (or all, use_filter = 0) go to the exact kernel, zero-volume
+// ones are counted; rows the filter cannot certify go to the row queue, as in the span kernel.
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <cmath>
 
 #include "voxtet.h"
 #include "tet_math.cuh"
@@ -42,18 +44,18 @@ namespace voxtet {
 constexpr int kSuWarps = kSuBlock / 32;
 constexpr int kSuBuckets = 64;                           // row counts 1..63 one bucket each, >= 64 together
 constexpr int kSuCounters = kSuBuckets * kSuWarps;       // bucket-major, one counter per warp of each bucket
-constexpr int kSuRec = 20;  // floats per tet record: 16 used; 5 groups of 16 bytes, an odd number,
-                            // so that lanes loading records of random slots spread over all banks
+constexpr int kSuRec = 20;  // floats per tet record: 5 groups of 16 bytes, an odd number, so that
+                            // lanes loading records of random slots spread over all banks
 constexpr int kSuStage = 64;                             // staged uncertain rows per block (about 5 per tile)
 constexpr uint32_t kSuEmpty = 0xFFFFFFFFu;               // a slice without candidate rows
 static_assert(kSuBlock == 128 && kSuSlices <= 32 && kSuRows == 1024, "unit fields: 7 + 5 bits; rows in 10 bits");
 
 // Tet record (kSuRec words per slot): alpha' of the four faces | beta | gamma | E of the upper
-// and of the lower side, i0 | (na - 1) << 16 | upper slots << 30, j0 | (l0 - z0) << 16.  Upper faces fill the slots from the
+// side (sign bit: slot 1 is an upper face) and of the lower side (sign bit: slot 2 is an upper
+// face), i0 | (na - 1) << 16, j0 | (l0 - z0) << 16 | the four faces' E.  Upper faces fill the slots from the
 // front and lower faces from the back; a face parallel to x leaves a neutral upper slot (alpha' =
 // +infinity) between them.  Slot 0 is always an upper face and slot 3 a lower one.
-constexpr int kRecB = 4, kRecG = 8, kRecEU = 12, kRecEL = 13, kRecX = 14, kRecYZ = 15;
-constexpr int kSuColumns = 1 << 14;  // most samples along x of a tet's box (14 bits hold na - 1)
+constexpr int kRecB = 4, kRecG = 8, kRecEU = 12, kRecEL = 13, kRecX = 14, kRecYZ = 15, kRecE = 16;
 
 // Shared memory of one block (dynamic), for tets of at most SL slices.
 template <int SL>
@@ -68,6 +70,8 @@ struct SuSmem {
   uint32_t warp_tot[kSuWarps];
   RowStageN<kSuStage> stage;
   long long tile;
+  int c0, r0;            // the current window: slices from c0, rows from r0 of each tet's box
+  int next_c0, next_r0;  // the window after it (0, 0: the tile is done)
 };
 
 // 16-slice tiles fit 7 blocks per SM (228 KB, 1 KB reserved per block), 32-slice tiles 5
@@ -79,12 +83,21 @@ __device__ __forceinline__ int su_counter(int n, int w) {
   return (kSuBuckets - min(n, kSuBuckets)) * kSuWarps + w;
 }
 
-// Phase (1) for tet t of this thread (t < 0: none).  Returns the slices whose entries it
-// wrote to sm.slice (0 if the tet has no unit here); counts each unit in its counter (no
-// rank is needed here, so the count does not wait on the shared-memory atomic).
-template <bool STRICT, bool CULL, int SL>
-__device__ __forceinline__ int su_setup(const Params &p, long long t, SuSmem<SL> &sm, TileCounters &ctr) {
+// Phase (1) for tet t of this thread's group (t < 0: none).  The group's 2^lg threads each set
+// the tet up and take its slices c0 + sub, c0 + sub + 2^lg, ... (sub = the thread within its
+// group), at most SL of them: a window of SL 2^lg slices from c0.  Returns the entries it wrote
+// to sm.slice (0 if none); counts each unit in its counter (no rank is needed here, so the
+// count does not wait on the shared-memory atomic).  `more` is set if the tet has slices past
+// the window; a window also covers at most kSuRows rows per slice, from row r0 of the box, and
+// `tall` is set if the tet's box has rows past it.  A tet is counted (or queued) once, by its
+// group's first thread in its first window.
+template <bool STRICT, bool CULL, bool TALL, int SL>
+__device__ __forceinline__ int su_setup(const Params &p, long long t, int lg, SuSmem<SL> &sm, TileCounters &ctr,
+                                        bool &more, bool &tall) {
   const int tid = threadIdx.x, warp = tid >> 5;
+  const int sub = tid & ((1 << lg) - 1);
+  const int c0 = sm.c0, r0 = TALL ? sm.r0 : 0;
+  const bool first = (sub | c0 | r0) == 0;
   if (t < 0) return 0;
   int3 V[4];
   if (!load_tet(p, t, V, ctr.err)) return 0;
@@ -92,6 +105,7 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, SuSmem<SL>
   const int E = tet_box(V, p.sh, p.rx, p.ry, p.z0, p.z1, bx);
   const bool empty = bx.na <= 0 || bx.nb <= 0 || bx.nc <= 0;
   if (E > kNarrowExtent) {  // wider than 2^20 lattice units: 128-bit sign, exact kernel
+    if (!first) return 0;
     if (v6_sign(V, E) == 0) {
       ++ctr.degenerate;
       return 0;
@@ -111,20 +125,17 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, SuSmem<SL>
   i64 n3x = (i64)e1y * e2z - (i64)e1z * e2y, n3y = (i64)e1z * e2x - (i64)e1x * e2z, n3z = (i64)e1x * e2y - (i64)e1y * e2x;
   i64 v6 = (i64)e1x * n1x + (i64)e1y * n1y + (i64)e1z * n1z;
   if (v6 == 0) {
-    ++ctr.degenerate;
+    ctr.degenerate += first;
     return 0;
   }
   if (empty) return 0;
   if (p.exact_all || bx.nb > kMaxFilterRows) {
+    if (!first) return 0;
     const unsigned k = atomicAdd(&p.hdr->tetq_count, 1u);
     p.tetq[k] = (uint32_t)t;
     return 0;
   }
-  if (bx.nc > SL || bx.nb > kSuRows || bx.na > kSuColumns) {  // the span kernel takes it (list mode)
-    const unsigned k = atomicAdd(&p.hdr->listq_count, 1u);
-    p.tetq[p.n_tets - 1 - k] = (uint32_t)t;
-    return 0;
-  }
+  tall = TALL && bx.nb > r0 + kSuRows;
   // Orientation (Lemma 1.1): for V6 < 0 every orientation value of an inside point is <= 0,
   // so negating the normals (and V6) gives the positively oriented form of the same faces.
   if (v6 < 0) {
@@ -173,6 +184,7 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, SuSmem<SL>
       rec[o] = a;
       rec[kRecB + o] = b;
       rec[kRecG + o] = g;
+      rec[kRecE + o] = e;
     } else {
       const i64 Dy = Ny[m] << p.sh, Dz = Nz[m] << p.sh;
       if (nz == 0) {
@@ -187,10 +199,11 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, SuSmem<SL>
     rec[cu] = __int_as_float(0x7f800000);
     rec[kRecB + cu] = 0.f;
     rec[kRecG + cu] = 0.f;
+    rec[kRecE + cu] = 0.f;
   }
-  rec[kRecEU] = eU;
-  rec[kRecEL] = eL;
-  rec[kRecX] = __uint_as_float((uint32_t)bx.i0 | ((uint32_t)(bx.na - 1) << 16) | ((uint32_t)cu << 30));
+  rec[kRecEU] = __int_as_float(__float_as_int(eU) | (cu >= 2 ? (int)0x80000000 : 0));
+  rec[kRecEL] = __int_as_float(__float_as_int(eL) | (cu >= 3 ? (int)0x80000000 : 0));
+  rec[kRecX] = __uint_as_float((uint32_t)bx.i0 | ((uint32_t)(bx.na - 1) << 16));
   rec[kRecYZ] = __uint_as_float((uint32_t)bx.j0 | ((uint32_t)(bx.l0 - p.z0) << 16));
   // Candidate rows of each slice: the cross-section's y-extent (a superset of the rows with
   // samples), narrowed exactly by the faces parallel to x.  Each unit is counted (no rank is
@@ -203,28 +216,33 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, SuSmem<SL>
     R.aL0 = R.aL1 = 0.f;
     R.aU0 = R.aU1 = fb;
   }
-  int units = 0;
-  float cf = 0.f;
-  for (int k = 0; k < bx.nc; ++k, cf += 1.f) {
+  const float row0 = (float)r0, row1 = TALL ? fminf(fb, (float)(r0 + kSuRows - 1)) : fb;
+  const uint32_t row0_bits = kMagicBits + (uint32_t)r0;
+  const int step = 1 << lg, k_end = min(bx.nc, c0 + (SL << lg));
+  more = bx.nc > k_end;
+  int units = 0, kk = 0;
+  float cf = (float)(c0 + sub);
+  const float cstep = (float)step;
+  for (int k = c0 + sub; k < k_end; k += step, cf += cstep, ++kk) {
     float flo, fhi;
-    slice_range(R, cf, fb, flo, fhi);
+    slice_range(R, cf, row0, row1, flo, fhi);
     bool any = flo <= fhi;
-    uint32_t b_lo = __float_as_uint(flo) - kMagicBits, n1 = __float_as_uint(fhi) - __float_as_uint(flo);
+    uint32_t b_lo = __float_as_uint(flo) - row0_bits, n1 = __float_as_uint(fhi) - __float_as_uint(flo);
     if (nz > 0 && any) {
-      int lo = (int)b_lo, hi = (int)(b_lo + n1);
+      int lo = (int)b_lo + r0, hi = lo + (int)n1;
       narrow_by_row_constraint<STRICT>(zL0 + zDz0 * (i64)k, zDy0, lo, hi);
       if (nz > 1) narrow_by_row_constraint<STRICT>(zL1 + zDz1 * (i64)k, zDy1, lo, hi);
       any = lo <= hi;
-      b_lo = (uint32_t)lo;
+      b_lo = (uint32_t)(lo - r0);
       n1 = (uint32_t)(hi - lo);
     }
     if (any) {
       atomicAdd(&sm.hist[su_counter((int)n1 + 1, warp)], 1u);
       ++units;
     }
-    sm.slice[k][tid] = any ? b_lo | (n1 << 10) : kSuEmpty;
+    sm.slice[kk][tid] = any ? b_lo | (n1 << 10) : kSuEmpty;
   }
-  return units ? bx.nc : 0;
+  return units ? kk : 0;
 }
 
 // Block-wide exclusive prefix sum of one value per thread (all threads call it); `total`
@@ -252,15 +270,21 @@ __device__ __forceinline__ uint32_t su_block_scan(SuSmem<SL> &sm, uint32_t v, ui
   return before;
 }
 
-// Phase (3): rows b0 .. b0 + n - 1 of slice k of the tet in `slot` (tet index t).
-template <bool STRICT, bool CLAMP, int SL>
+// The tet at place i of a launch (below `end`, else -1): tet i, or the i-th listed one.
+template <bool LIST>
+__device__ __forceinline__ long long su_tet(const Params &p, long long i, long long end) {
+  if (i >= end) return -1;
+  return LIST ? (long long)p.tetq[p.n_tets - 1 - i] : i;
+}
+
+// Phase (3): rows b0 .. b0 + n - 1 of slice k of the tet in `slot` (place t of the launch).
+template <bool STRICT, bool CLAMP, bool LIST, bool BATCH, int SL>
 __device__ __forceinline__ void su_walk(const Params &p, SuSmem<SL> &sm, int slot, long long t, int k, int b0, int n) {
   const float4 *R = reinterpret_cast<const float4 *>(sm.rec + slot * kSuRec);
   const float4 qa = R[0], qb = R[1], qg = R[2], qi = R[3];
   const float cf = (float)k, INF = __int_as_float(0x7f800000);
   const uint32_t xx = __float_as_uint(qi.z), yz = __float_as_uint(qi.w);
-  const uint32_t nup = xx >> 30;
-  const bool up1 = nup >= 2, up2 = nup >= 3;
+  const bool up1 = __float_as_int(qi.x) < 0, up2 = __float_as_int(qi.y) < 0;
   const float a1 = __fmaf_rn(qg.y, cf, qa.y), a2 = __fmaf_rn(qg.z, cf, qa.z);
   RowFaces f;
   f.aU0 = __fmaf_rn(qg.x, cf, qa.x);
@@ -275,9 +299,9 @@ __device__ __forceinline__ void su_walk(const Params &p, SuSmem<SL> &sm, int slo
   f.bL1 = up1 ? 0.f : qb.y;
   f.aL2 = up2 ? -INF : a2;
   f.bL2 = up2 ? 0.f : qb.z;
-  f.eU = qi.x;
-  f.eL = qi.y;
-  row_magic<STRICT>(f, (int)(xx & 0xFFFFu), (int)((xx >> 16) & 0x3FFFu));
+  f.eU = fabsf(qi.x);
+  f.eL = fabsf(qi.y);
+  row_magic<STRICT>(f, (int)(xx & 0xFFFFu), (int)(xx >> 16));
   // rows of the slab from its first: below 2^32 for every accepted grid
   const uint32_t r0 = ((yz >> 16) + (uint32_t)k) * (uint32_t)p.ry + (yz & 0xFFFFu) + (uint32_t)b0;
   uint32_t *const row = p.out + (size_t)r0 * (uint32_t)p.W - kMagicWord;
@@ -288,86 +312,195 @@ __device__ __forceinline__ void su_walk(const Params &p, SuSmem<SL> &sm, int slo
   for (int s0 = 0; s0 < n; s0 += 32) {
     const int s1 = min(n, s0 + 32);
     uint32_t amb = 0;
-    for (int r = s0; r < s1; ++r) {
+    const float b_end = bf + (float)(s1 - s0);
+#pragma unroll 1
+    do {
       uint32_t lo, hi;
       bool live;
-      amb |= (uint32_t)row_bounds<STRICT, CLAMP>(f, bf, lo, hi, live) << (r - s0);
-      row_or(row, off, lo, hi, live);
+      bool a = row_bounds<STRICT, CLAMP>(f, bf, lo, hi, live);
+      if (a) {
+        a = row_refine<STRICT>(f, R[kRecE / 4], up1, up2, bf);
+        live = !a && __uint_as_float(lo) <= __uint_as_float(hi);
+      }
+      amb = amb + amb + (a ? 1u : 0u);  // the last row in the lowest bit
+      row_or<BATCH>(row, off, lo, hi, live);
       bf += 1.f;
       off += (uint32_t)p.W;
-    }
+    } while (bf != b_end);
     while (amb) {
       const int j = __ffs(amb) - 1;
       amb &= amb - 1u;
-      queue_row_staged(p, sm.stage, t, b0 + s0 + j, k);
+      queue_row_staged(p, sm.stage, su_tet<LIST>(p, t, p.n_tets), b0 + s1 - 1 - j, k);
     }
   }
 }
 
-template <bool STRICT, bool CULL, bool CLAMP, bool STRIDED, int SL>
+// Phases (1)-(3) of one window of a tile: the tets at places base .. base + (kSuBlock >> lg) - 1
+// (those below `end`), each shared by a group of 2^lg threads.  All threads of the block call it,
+// in step.  The caller's
+// loop claims a tile or moves to the tile's next window: a loop of its own around these phases
+// cost the row loop its reconvergence (measured on GB300, sliver mesh at 512^3: 26.7 -> 15.9
+// active lanes, 262 -> 440 us).
+template <bool STRICT, bool CULL, bool CLAMP, bool TALL, bool LIST, bool BATCH, int SL>
+__device__ __forceinline__ void su_pass(const Params &p, long long base, long long end, int lg, SuSmem<SL> &sm,
+                                        TileCounters &ctr) {
+  const int tid = threadIdx.x;
+  // (1) set up this thread's tet and its slices' row ranges; count units per counter
+  bool more = false, tall = false;
+  const long long t = su_tet<LIST>(p, base + (tid >> lg), end);
+  const int nc = su_setup<STRICT, CULL, TALL, SL>(p, t, lg, sm, ctr, more, tall);
+  {
+    const bool any_more = __syncthreads_or(more);
+    const bool any_tall = TALL && p.ry > kSuRows && __syncthreads_or(tall);
+    if (tid == 0) {  // every slice of these rows first, then the next rows
+      sm.next_c0 = any_more ? sm.c0 + (SL << lg) : 0;
+      if (TALL) sm.next_r0 = any_more ? sm.r0 : any_tall ? sm.r0 + kSuRows : 0;
+    }
+  }
+  // (2) exclusive scan of the counters (two per thread) into cursors, then every unit to
+  // its place (a cursor per counter: units of one counter come from one warp)
+  {
+    const uint32_t h0 = sm.hist[2 * tid], h1 = sm.hist[2 * tid + 1];
+    uint32_t all = 0;
+    const uint32_t before = su_block_scan(sm, h0 + h1, all);
+    sm.hist[2 * tid] = before;
+    sm.hist[2 * tid + 1] = before + h0;
+    if (tid == 0) sm.total = all;
+    __syncthreads();
+  }
+  const uint32_t total = sm.total;
+#pragma unroll 4
+  for (int k = 0; k < nc; ++k) {
+    const uint32_t e = sm.slice[k][tid];
+    if (e == kSuEmpty) continue;
+    const int n = (int)(e >> 10) + 1;
+    const uint32_t pos = atomicAdd(&sm.hist[su_counter(n, tid >> 5)], 1u);
+    sm.unit[pos] = (uint32_t)tid | ((uint32_t)k << 7) | (e << 12);
+  }
+  __syncthreads();
+  if (tid == 0) ctr.spans += total;
+  sm.hist[2 * tid] = 0u;  // ready for the next tile's counts (a barrier comes before them)
+  sm.hist[2 * tid + 1] = 0u;
+  // (3) walk the units, longest first; a warp takes 32 neighbouring units of the order
+  const int c0 = sm.c0, r0 = TALL ? sm.r0 : 0;
+  for (uint32_t i = tid; i < total; i += kSuBlock) {
+    const uint32_t u = sm.unit[i];
+    const int slot = (int)(u & 127u);
+    const int k = c0 + ((int)((u >> 7) & 31u) << lg) + (slot & ((1 << lg) - 1));
+    const int b0 = (int)((u >> 12) & 1023u) + r0, n = (int)(u >> 22) + 1;
+    ctr.rows += (unsigned)n;
+    su_walk<STRICT, CLAMP, LIST, BATCH, SL>(p, sm, slot, base + (slot >> lg), k, b0, n);
+  }
+  flush_stage(p, sm.stage);
+}
+
+// The block's first thread moves to the tile's next window; true if the tile is done and
+// another is to be claimed.
+template <int SL>
+__device__ __forceinline__ bool su_next_window(SuSmem<SL> &sm) {
+  sm.c0 = sm.next_c0;
+  sm.r0 = sm.next_r0;
+  return (sm.c0 | sm.r0) == 0;
+}
+
+template <int SL>
+__device__ __forceinline__ void su_begin(SuSmem<SL> &sm) {
+  for (int i = threadIdx.x; i < kSuCounters; i += kSuBlock) sm.hist[i] = 0u;
+  if (threadIdx.x == 0) {
+    sm.stage.n = 0;
+    sm.next_c0 = sm.next_r0 = 0;
+  }
+}
+
+// Should twice as many threads share a tet as 2^lg, for tiles of about even work over `blocks`
+// resident blocks: `tiles` now, `rows` a tet.  Every thread repeats the tet's setup, about 20 rows'
+// worth: up to two tiles a block if that adds a fifth, up to four if it adds a twentieth.  Measured
+// on GB300: a 4096^3 torus of 198,529 tets in slabs of 64 slices 7.1 ms without, 4.4 up to two
+// tiles, 4.2 up to four; 196,608 tets at 512^3 144 -> 133 us; but a 30-slice slab of 50 rows a tet 56
+// -> 61 us where the added setup is not looked at.
+static __host__ __device__ __forceinline__ bool su_share_more(long long tiles, long long blocks, float rows, int lg) {
+  const float added = 20.0f * (float)((2 << lg) - 1);
+  return (tiles < 2 * blocks && 5.0f * added <= rows) || (tiles < 4 * blocks && 20.0f * added <= rows);
+}
+
+// LIST: the tets are the hdr->listq_count ones listed at the back of p.tetq.
+template <bool STRICT, bool CULL, bool CLAMP, bool LIST, int SL>
 __global__ void __launch_bounds__(kSuBlock, SL == kSuSlicesSmall ? 7 : 5) k_slices(Params p) {
-  chain_wait();  // vertices snapped, header zeroed
+  chain_wait();  // vertices snapped, header zeroed, tets listed
   chain_release();
   extern __shared__ __align__(16) unsigned char su_dyn_smem[];
   SuSmem<SL> &sm = *reinterpret_cast<SuSmem<SL> *>(su_dyn_smem);
-  const int tid = threadIdx.x;
   TileCounters ctr;
-  for (int i = tid; i < kSuCounters; i += kSuBlock) sm.hist[i] = 0u;
-  if (tid == 0) sm.stage.n = 0;
+  su_begin(sm);
+  const long long end = LIST ? (long long)p.hdr->listq_count : p.n_tets;
+  int lg = p.lg;
+  if (LIST && end > 0) {  // as su_group_log2, with the slab's tets counted and their rows added up
+    const float slab = (float)(p.z1 - p.z0), rows = 0.5f * (float)p.hdr->list_rows / (float)end;
+    while (lg < kSuMaxGroup && (float)(1 << lg) < slab &&
+           (((end << lg) / kSuBlock) * 2 < (long long)gridDim.x ||
+            su_share_more((end << lg) / kSuBlock, (long long)gridDim.x, rows, lg)))
+      ++lg;
+  }
   for (;;) {
-    if (tid == 0) sm.tile = (long long)atomicAdd(&p.hdr->tile_counter, 1ull);
+    if (threadIdx.x == 0 && su_next_window(sm)) sm.tile = (long long)atomicAdd(&p.hdr->tile_counter, 1ull);
     __syncthreads();
-    const long long tile = sm.tile;
-    long long base, t;
-    if (STRIDED) {  // slab launches: tile k holds tets k + j * tile_stride
-      if (tile >= p.tile_stride) break;
-      base = tile;
-      t = base + (long long)tid * p.tile_stride;
-    } else {
-      base = tile * kSuBlock;
-      if (base >= p.n_tets) break;
-      t = base + tid;
-    }
-    if (t >= p.n_tets) t = -1;
-    // (1) set up this thread's tet and its slices' row ranges; count units per counter
-    const int nc = su_setup<STRICT, CULL, SL>(p, t, sm, ctr);
-    __syncthreads();
-    // (2) exclusive scan of the counters (two per thread) into cursors, then every unit to
-    // its place (a cursor per counter: units of one counter come from one warp)
-    {
-      const uint32_t c0 = sm.hist[2 * tid], c1 = sm.hist[2 * tid + 1];
-      uint32_t all = 0;
-      const uint32_t before = su_block_scan(sm, c0 + c1, all);
-      sm.hist[2 * tid] = before;
-      sm.hist[2 * tid + 1] = before + c0;
-      if (tid == 0) sm.total = all;
-      __syncthreads();
-    }
-    const uint32_t total = sm.total;
-#pragma unroll 4
-    for (int k = 0; k < nc; ++k) {
-      const uint32_t e = sm.slice[k][tid];
-      if (e == kSuEmpty) continue;
-      const int n = (int)(e >> 10) + 1;
-      const uint32_t pos = atomicAdd(&sm.hist[su_counter(n, tid >> 5)], 1u);
-      sm.unit[pos] = (uint32_t)tid | ((uint32_t)k << 7) | (e << 12);
-    }
-    __syncthreads();
-    if (tid == 0) ctr.spans += total;
-    sm.hist[2 * tid] = 0u;  // ready for the next tile's counts (a barrier comes before them)
-    sm.hist[2 * tid + 1] = 0u;
-    // (3) walk the units, longest first; a warp takes 32 neighbouring units of the order
-    for (uint32_t i = tid; i < total; i += kSuBlock) {
-      const uint32_t u = sm.unit[i];
-      const int slot = (int)(u & 127u), k = (int)((u >> 7) & 31u);
-      const int b0 = (int)((u >> 12) & 1023u), n = (int)(u >> 22) + 1;
-      const long long tt = STRIDED ? base + (long long)slot * p.tile_stride : base + slot;
-      ctr.rows += (unsigned)n;
-      su_walk<STRICT, CLAMP, SL>(p, sm, slot, tt, k, b0, n);
-    }
-    flush_stage(p, sm.stage);
+    const long long base = sm.tile * (kSuBlock >> lg);
+    if (base >= end) break;
+    su_pass<STRICT, CULL, CLAMP, SL == kSuSlices, LIST, false, SL>(p, base, end, lg, sm, ctr);
   }
   flush_counters(p.hdr, ctr);
+}
+
+// The tiles of every job of a batch, claimed from one counter; a tile's job is found in the
+// per-job tile offsets by one warp.  A job's device-detected errors also go to its status word.
+template <bool STRICT, bool CULL>
+__global__ void __launch_bounds__(kSuBlock, 7) k_slices_batched(BatchHeader *bh, const JobDesc *jobs,
+                                                               const unsigned long long *tile_base, int *status) {
+  chain_wait();  // vertices snapped, headers and grids zeroed
+  chain_release();
+  constexpr int SL = kSuSlicesSmall;
+  extern __shared__ __align__(16) unsigned char su_dyn_smem[];
+  SuSmem<SL> &sm = *reinterpret_cast<SuSmem<SL> *>(su_dyn_smem);
+  __shared__ Params sp;
+  __shared__ int job_s;
+  const int tid = threadIdx.x;
+  TileCounters ctr;
+  su_begin(sm);
+  const int n = bh->n_jobs;
+  const unsigned long long total = bh->total_tiles;
+  int cur = -1;
+  for (;;) {
+    if (tid < 32) {
+      unsigned long long tile = 0;
+      int claim = 0;
+      if (tid == 0) {
+        claim = su_next_window(sm);
+        if (claim) tile = atomicAdd(&bh->tile_counter, 1ull);
+      }
+      claim = __shfl_sync(0xFFFFFFFFu, claim, 0);
+      if (claim) {
+        tile = __shfl_sync(0xFFFFFFFFu, tile, 0);
+        const int j = tile < total ? find_job_warp(tile_base, n, tile) : -1;
+        if (tid == 0) {
+          sm.tile = j < 0 ? 0 : (long long)(tile - tile_base[j]);
+          job_s = j;
+        }
+      }
+    }
+    __syncthreads();
+    const int j = job_s;
+    if (j < 0) break;
+    if (j != cur) {  // a new job: flush the previous job's counters, load its Params
+      if (cur >= 0) flush_counters(sp.hdr, ctr, status + cur);
+      __syncthreads();
+      if (tid < (int)(sizeof(Params) / sizeof(uint32_t)))
+        reinterpret_cast<uint32_t *>(&sp)[tid] = reinterpret_cast<const uint32_t *>(&jobs[j].p)[tid];
+      __syncthreads();
+      cur = j;
+    }
+    su_pass<STRICT, CULL, false, true, false, true, SL>(sp, sm.tile * (kSuBlock >> sp.lg), sp.n_tets, sp.lg, sm, ctr);
+  }
+  if (cur >= 0) flush_counters(sp.hdr, ctr, status + cur);
 }
 
 // ------------------------------------------------------------------ host side
@@ -404,6 +537,56 @@ size_t slices_smem_bytes(int slices) {
   return slices <= kSuSlicesSmall ? sizeof(SuSmem<kSuSlicesSmall>) : sizeof(SuSmem<kSuSlices>);
 }
 
+int su_group_log2(long long n_tets, int side, int slab, int slices, long long blocks) {
+  if (n_tets < 1) return 0;
+  const double w = (double)side / std::cbrt((double)n_tets / 6.0);
+  const double span = w < slab ? w : slab;  // slices a tet spans, about
+  int lg = 0;
+  while (lg < kSuMaxGroup && (double)(slices << lg) < span) ++lg;
+  while (lg < kSuMaxGroup && (double)(1 << lg) < span && ((n_tets << lg) / kSuBlock) * 2 < blocks) ++lg;
+  while (lg < kSuMaxGroup && (double)(1 << lg) < span &&
+         su_share_more((n_tets << lg) / kSuBlock, blocks, (float)(0.5 * w * span), lg))
+    ++lg;
+  return lg;
+}
+
+typedef void (*SuBatchKernel)(BatchHeader *, const JobDesc *, const unsigned long long *, int *);
+
+static SuBatchKernel su_batch_kernel(bool strict, bool cull) {
+  if (strict) return cull ? k_slices_batched<true, true> : k_slices_batched<true, false>;
+  return cull ? k_slices_batched<false, true> : k_slices_batched<false, false>;
+}
+
+static int g_su_batch_occ[kSuMaxDevices][4];
+
+int slices_batched_blocks(bool strict, bool cull) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kSuMaxDevices) return 0;
+  int &slot = g_su_batch_occ[dev][(strict ? 2 : 0) | (cull ? 1 : 0)];
+  if (slot == 0) {
+    while (g_su_lock.exchange(1)) {
+    }
+    const SuBatchKernel kern = su_batch_kernel(strict, cull);
+    const size_t smem = slices_smem_bytes(kSuSlicesSmall);
+    int occ = 0;
+    cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(kern),
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kSuBlock, smem);
+    if (e == cudaSuccess) slot = occ > 0 ? occ : 1;
+    g_su_lock.store(0);
+  }
+  return slot;
+}
+
+int launch_slices_batched(BatchHeader *bh, const JobDesc *jobs, const unsigned long long *tile_base, int *status,
+                          bool strict, bool cull, int sms, cudaStream_t stream) {
+  const int occ = slices_batched_blocks(strict, cull);
+  if (occ < 1) return VOXTET_ERR_CUDA;
+  const cudaError_t e = launch_chained(su_batch_kernel(strict, cull), (unsigned)(sms * occ), kSuBlock,
+                                       slices_smem_bytes(kSuSlicesSmall), stream, bh, jobs, tile_base, status);
+  return e == cudaSuccess ? VOXTET_OK : VOXTET_ERR_CUDA;
+}
+
 int launch_slices(const Params &p_in, int variant, int slices, int sms, cudaStream_t stream) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kSuMaxDevices) return VOXTET_ERR_CUDA;
@@ -423,16 +606,13 @@ int launch_slices(const Params &p_in, int variant, int slices, int sms, cudaStre
     if (e != cudaSuccess) return VOXTET_ERR_CUDA;
   }
   Params p = p_in;
-  const bool strided = (variant & 8) != 0;
+  const bool list = (variant & 8) != 0;
   long long grid = (long long)sms * occ;
-  long long tiles = (p.n_tets + kSuBlock - 1) / kSuBlock;
-  p.tile_stride = 0;
-  if (strided) {  // at least one tile per resident block (see the span kernel's slab launches)
-    long long stride = tiles;
-    if (stride < grid) stride = p.n_tets < grid ? p.n_tets : grid;
-    p.tile_stride = stride;
-    tiles = stride;
-  }
+  // a list's length is known on the device only: the kernel shares its tets among more threads
+  const int side = 1 << (kLatticeBits - p.sh);
+  p.lg = list ? 0 : su_group_log2(p.n_tets, side, p.z1 - p.z0, slices, grid);
+  const int per_tile = kSuBlock >> p.lg;
+  const long long tiles = list ? grid : (p.n_tets + per_tile - 1) / per_tile;
   if (grid > tiles) grid = tiles;
   if (grid < 1) grid = 1;
   return launch_chained(kern, (unsigned)grid, kSuBlock, smem, stream, p) == cudaSuccess ? VOXTET_OK : VOXTET_ERR_CUDA;

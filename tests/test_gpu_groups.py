@@ -1,0 +1,140 @@
+"""Slice units shared by groups of threads, taken in windows, listed per slab and batched: where a tet's
+slices and rows exceed one window, and where few or wide tets are shared by many threads.  All bit for
+bit against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2106_01326_gb300 import meshgen as mg
+
+pytestmark = pytest.mark.gpu
+
+L = 1 << 20
+
+
+@pytest.fixture(scope="module")
+def vt():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    from paper_2106_01326_gb300 import build as vbuild
+    from paper_2106_01326_gb300 import voxtet
+
+    vbuild.build()
+    oracle.build()
+    voxtet.load()
+    return voxtet
+
+
+def _cuda(verts, tets):
+    import torch
+
+    return torch.from_numpy(np.ascontiguousarray(verts)).cuda(), torch.from_numpy(np.ascontiguousarray(tets)).cuda()
+
+
+def _soup(seed, n, res, lo, hi, axis_scale=(1.0, 1.0, 1.0)):
+    """n tets of lo..hi voxels (times axis_scale) anywhere in the unit cube, some flat or inverted."""
+    rng = np.random.default_rng(seed)
+    o = rng.random((n, 1, 3))
+    size = np.exp(rng.uniform(np.log(lo), np.log(hi), size=(n, 1, 1))) / res * np.asarray(axis_scale)
+    v = (o + (rng.random((n, 4, 3)) - 0.5) * size).astype(np.float32)
+    v[8::17, 3] = v[8::17, 2]  # zero volume
+    return v.reshape(-1, 3), np.arange(4 * n, dtype=np.int32).reshape(n, 4)
+
+
+def _same(got, ref, what):
+    got = got.cpu().numpy().view(np.uint32)
+    assert np.array_equal(got.reshape(ref.shape), ref), what
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("n,res,lo,hi", [(1, 128, 90, 120), (3, 256, 60, 200), (40, 128, 1, 100), (700, 64, 1, 60),
+                                         (5000, 128, 1, 8), (20000, 64, 0.5, 20), (140000, 32, 0.3, 3)])
+def test_groups_and_windows(vt, n, res, lo, hi, mode):
+    """From one tet (a whole block shares it) to meshes with a thread a tet, in both cases with tets of
+    more slices than a window holds."""
+    verts, tets = _soup(n, n, res, lo, hi)
+    ref = oracle.voxelize(verts, tets, (0, 0, 0), 1.0 / res, res, mode=mode)
+    v, t = _cuda(verts, tets)
+    _same(vt.voxelize(v, t, (0, 0, 0), 1.0 / res, res, mode=mode), ref, "culled")
+    _same(vt.voxelize(v, t, (0, 0, 0), 1.0 / res, res, mode=mode, row_cull=2), ref, "all rows")
+
+
+@pytest.mark.parametrize("dims,scale", [((40, 2100, 24), (0.2, 2, 0.2)), ((17, 1030, 9), (0.3, 2.1, 0.3)),
+                                        ((5000, 20, 12), (2, 0.3, 0.3)), ((9, 12, 1200), (0.3, 0.3, 2))])
+def test_more_rows_and_columns_than_a_window(vt, dims, scale):
+    """Boxes of more than 1024 rows per slice, of thousands of columns, and of 1200 slices."""
+    h = 1.0 / 64
+    verts, tets = _soup(3, 300, 64, 4, 30, scale)
+    verts = verts * np.array([dims[0] * h, dims[1] * h, dims[2] * h], dtype=np.float32)
+    ref = oracle.voxelize_grid(verts, tets, (0, 0, 0), h, dims)
+    v, t = _cuda(verts, tets)
+    _same(vt.voxelize_grid(v, t, (0, 0, 0), h, dims), ref, dims)
+
+
+@pytest.mark.parametrize("z0,z1", [(0, 1), (31, 33), (40, 52), (99, 100), (60, 72)])
+@pytest.mark.parametrize("n,lo,hi", [(50, 5, 90), (9000, 1, 6)])
+def test_thin_slab_lists(vt, n, lo, hi, z0, z1):
+    """Slabs below an eighth of the grid go through the list of their tets; tets wider than the exact
+    integers of the filter path go to the exact kernel from there, flat ones are only counted."""
+    dims, h = (90, 70, 100), 1.0 / 128
+    verts, tets = _soup(n, n, 128, lo, hi)
+    wide = np.array([[-0.9, -0.9, -0.5], [1.9, 0.1, 0.4], [0.2, 1.9, 0.6], [0.3, 0.4, 1.7]], dtype=np.float32)
+    tets = np.concatenate([tets, [[len(verts) + k for k in range(4)]]]).astype(np.int32)
+    verts = np.concatenate([verts, wide])
+    ref = oracle.voxelize_grid(verts, tets, (0, 0, 0), h, dims, z0=z0, z1=z1)
+    v, t = _cuda(verts, tets)
+    ws = vt.alloc_workspace(len(tets), len(verts), 100)
+    _same(vt.voxelize_grid(v, t, (0, 0, 0), h, dims, z_range=(z0, z1), workspace=ws), ref, (z0, z1))
+    st = vt.read_stats(ws)
+    assert st["wide_tets"] == 1 and st["degenerate_tets"] >= len(range(8, n, 17))
+    bad = tets.copy()
+    bad[len(bad) // 2, 1] = len(verts)
+    st, _ = vt.voxelize_grid(v, _cuda(verts, bad)[1], (0, 0, 0), h, dims, z_range=(z0, z1), raise_on_error=False)
+    assert st == vt.ERR_INDEX
+
+
+@pytest.mark.parametrize("n,res", [(4, 256), (6, 256)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_wide_tets_few_rows_left_to_the_exact_kernels(vt, n, res, mode):
+    """Tets of 43 and 64 voxels: a steep face's error would give up most of a tet's rows if it stood
+    for the whole side; with each face's own error few are left."""
+    verts, tets = mg.kuhn_lattice(n, jitter=0.25, seed=11)
+    verts, tets = verts.astype(np.float32), tets.astype(np.int32)
+    ref = oracle.voxelize(verts, tets, (0, 0, 0), 1.0 / res, res, mode=mode)
+    v, t = _cuda(verts, tets)
+    ws = vt.alloc_workspace(len(tets), len(verts), res)
+    _same(vt.voxelize(v, t, (0, 0, 0), 1.0 / res, res, mode=mode, workspace=ws), ref, (n, res))
+    st = vt.read_stats(ws)
+    assert st["fallback_rows"] < 0.01 * st["rows"], st
+
+
+def test_batch_of_unlike_jobs(vt):
+    """One batch with jobs of one tet, of wide tets, of many small ones, without tets, in lattice
+    coordinates and with an unaligned grid; each job's grid and status are its own."""
+    import torch
+
+    from paper_2106_01326_gb300 import batch
+
+    specs, refs = [], []
+    store = torch.full((1 << 20,), -1, dtype=torch.int32, device="cuda")
+    at = 1  # grids start on 4-byte boundaries only
+    for seed, n, res, lo, hi in ((1, 1, 64, 30, 60), (2, 300, 128, 10, 120), (3, 30000, 32, 0.3, 4), (4, 0, 64, 1, 2),
+                                 (5, 900, 64, 1, 50), (6, 129, 1, 0.5, 1), (7, 4000, 128, 1, 9)):
+        verts, tets = _soup(seed, n, res, lo, hi) if n else (np.zeros((0, 3), np.float32), np.zeros((0, 4), np.int32))
+        v, t = _cuda(verts, tets)
+        w = vt.grid_words(res)
+        specs.append(batch.JobSpec(batch.Mesh(v, t), res, store[at:at + w].view(res, res, -1)))
+        at += w
+        refs.append(oracle.voxelize(verts, tets, (0, 0, 0), 1.0 / res, res) if n else np.zeros((res, res, (res + 31) // 32), np.uint32))
+    bad = _soup(8, 60, 64, 1, 9)
+    bad_v = bad[0].copy()
+    bad_v[7, 1] = np.nan
+    v, t = _cuda(bad_v, bad[1])
+    specs.append(batch.JobSpec(batch.Mesh(v, t), 64, store[at:at + vt.grid_words(64)].view(64, 64, -1)))
+    for _ in range(2):
+        assert batch.voxelize_batched(specs) == [vt.OK] * len(refs) + [vt.ERR_NAN]
+        for k, (sp, ref) in enumerate(zip(specs, refs)):
+            _same(sp.out, ref, k)
+    assert int(store[0]) == -1 and int(store[at + vt.grid_words(64)]) == -1
