@@ -611,6 +611,8 @@ __device__ __forceinline__ void process_tile(const Params &p, long long base, lo
     ctr.rows += run_span<STRICT, CULL, CLAMP>(p, t, V, bx, c0, min(c0 + S, bx.nc), slice_tab, sm.stage, (mt & 1u) != 0);
   }
   flush_stage(p, sm.stage);
+  __syncthreads();
+  if (threadIdx.x == 0) sm.stage.n = 0;
 }
 
 // The slice table lives in dynamic shared memory: p.max_slices rows of kBlock words.
@@ -1673,7 +1675,7 @@ static size_t build_batch_image(const voxtet_job *jobs, int n, int cap, const vo
     d.p.W = (res + 31) / 32;
     d.p.sh = kLatticeBits - k;
     d.p.exact_all = o.use_filter ? 0 : 1;
-    d.p.lg = su_group_log2(nt, res, res, kSuSlicesSmall, (long long)(per_tet * (double)nt));
+    d.p.lg = su_group_log2(nt, res, res, res, kSuSlicesSmall, (long long)(per_tet * (double)nt));
     d.verts = J.d_verts;
     d.fixed = J.fixed_point ? 1 : 0;
     if (ok[j] && !J.fixed_point) d.s = snap_args(J.origin, J.voxel_size, k);
@@ -1692,6 +1694,10 @@ static size_t build_batch_image(const voxtet_job *jobs, int n, int cap, const vo
   bh->total_tiles = tsum;
   bh->total_prep = psum;
   bh->tile_counter = 0;
+  // neighbouring tiles mostly share a job, so a claim of several spares the search and the load of
+  // its Params; about eight claims a block keep the end even
+  const unsigned long long c = blocks > 0 ? tsum / (unsigned long long)(blocks * 8) : 1ull;
+  bh->chunk = c < 1 ? 1ull : c > 8 ? 8ull : c;
   return need;
 }
 

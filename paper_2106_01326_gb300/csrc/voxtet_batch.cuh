@@ -29,7 +29,8 @@ struct BatchHeader {
   unsigned long long total_tiles;
   unsigned long long total_prep;  // chunks of zeroing and snapping
   unsigned long long tile_counter;
-  unsigned long long reserved[28];
+  unsigned long long chunk;  // tiles a block claims at a time
+  unsigned long long reserved[27];
 };
 static_assert(sizeof(BatchHeader) == 256, "batch header is 256 bytes");
 

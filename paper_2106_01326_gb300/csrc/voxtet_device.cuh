@@ -313,7 +313,8 @@ __device__ __forceinline__ void queue_row_staged(const Params &p, RowStageN<N> &
   }
 }
 
-// Moves a block's staged rows to the global queue (all threads of the block call it).
+// Moves a block's staged rows to the global queue (all threads of the block call it).  The stage's
+// count is left for the caller to reset, after its next barrier.
 template <int N>
 __device__ __forceinline__ void flush_stage(const Params &p, RowStageN<N> &st) {
   __syncthreads();
@@ -328,8 +329,6 @@ __device__ __forceinline__ void flush_stage(const Params &p, RowStageN<N> &st) {
       else atomicOr(&p.redo[it.tet >> 5], 1u << (it.tet & 31));
     }
   }
-  __syncthreads();
-  if (threadIdx.x == 0) st.n = 0;
 }
 
 // Exact conversion of an integral float in [0, 2^22) to int without the conversion

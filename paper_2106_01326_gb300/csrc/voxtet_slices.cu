@@ -66,7 +66,6 @@ struct SuSmem {
   // the tile's units sorted by row count, longest first: slot | k << 7 | b_lo << 12 | (n - 1) << 22
   uint32_t unit[kSuBlock * SL];
   uint32_t hist[kSuCounters];  // unit counts, then (after the scan) cursors
-  uint32_t total;
   uint32_t warp_tot[kSuWarps];
   RowStageN<kSuStage> stage;
   long long tile;
@@ -246,7 +245,7 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, int lg, Su
 }
 
 // Block-wide exclusive prefix sum of one value per thread (all threads call it); `total`
-// gets the sum.  Uses sm.warp_tot; ends with the block in step.
+// gets the sum.  Uses sm.warp_tot, which no thread may write again before the next barrier.
 template <int SL>
 __device__ __forceinline__ uint32_t su_block_scan(SuSmem<SL> &sm, uint32_t v, uint32_t &total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -266,7 +265,6 @@ __device__ __forceinline__ uint32_t su_block_scan(SuSmem<SL> &sm, uint32_t v, ui
     if (w < warp) before += t;
     total += t;
   }
-  __syncthreads();
   return before;
 }
 
@@ -352,23 +350,21 @@ __device__ __forceinline__ void su_pass(const Params &p, long long base, long lo
   {
     const bool any_more = __syncthreads_or(more);
     const bool any_tall = TALL && p.ry > kSuRows && __syncthreads_or(tall);
-    if (tid == 0) {  // every slice of these rows first, then the next rows
+    if (tid == 0) {
+      sm.stage.n = 0;  // flushed by the previous window; every thread has passed a barrier since
+      // every slice of these rows first, then the next rows
       sm.next_c0 = any_more ? sm.c0 + (SL << lg) : 0;
       if (TALL) sm.next_r0 = any_more ? sm.r0 : any_tall ? sm.r0 + kSuRows : 0;
     }
   }
   // (2) exclusive scan of the counters (two per thread) into cursors, then every unit to
   // its place (a cursor per counter: units of one counter come from one warp)
-  {
-    const uint32_t h0 = sm.hist[2 * tid], h1 = sm.hist[2 * tid + 1];
-    uint32_t all = 0;
-    const uint32_t before = su_block_scan(sm, h0 + h1, all);
-    sm.hist[2 * tid] = before;
-    sm.hist[2 * tid + 1] = before + h0;
-    if (tid == 0) sm.total = all;
-    __syncthreads();
-  }
-  const uint32_t total = sm.total;
+  const uint32_t h0 = sm.hist[2 * tid], h1 = sm.hist[2 * tid + 1];
+  uint32_t total = 0;
+  const uint32_t before = su_block_scan(sm, h0 + h1, total);
+  sm.hist[2 * tid] = before;
+  sm.hist[2 * tid + 1] = before + h0;
+  __syncthreads();
 #pragma unroll 4
   for (int k = 0; k < nc; ++k) {
     const uint32_t e = sm.slice[k][tid];
@@ -413,14 +409,13 @@ __device__ __forceinline__ void su_begin(SuSmem<SL> &sm) {
 }
 
 // Should twice as many threads share a tet as 2^lg, for tiles of about even work over `blocks`
-// resident blocks: `tiles` now, `rows` a tet.  Every thread repeats the tet's setup, about 20 rows'
-// worth: up to two tiles a block if that adds a fifth, up to four if it adds a twentieth.  Measured
-// on GB300: a 4096^3 torus of 198,529 tets in slabs of 64 slices 7.1 ms without, 4.4 up to two
-// tiles, 4.2 up to four; 196,608 tets at 512^3 144 -> 133 us; but a 30-slice slab of 50 rows a tet 56
-// -> 61 us where the added setup is not looked at.
+// resident blocks: `tiles` now, `rows` a tet.  Every thread repeats the tet's setup, about 10 rows'
+// worth: up to four tiles a block while that adds less than a fifth.  Measured on GB300: a 4096^3
+// torus of 198,529 tets in slabs of 64 slices 5.41, 4.59, 4.27 and 4.28 ms with 4, 8, 16 and 32 threads
+// a tet (875 to 7000 tiles for 760 blocks); 196,608 tets at 512^3 144 -> 133 us with two; but a
+// 30-slice slab of about 50 rows a tet 56 -> 61 us with two.
 static __host__ __device__ __forceinline__ bool su_share_more(long long tiles, long long blocks, float rows, int lg) {
-  const float added = 20.0f * (float)((2 << lg) - 1);
-  return (tiles < 2 * blocks && 5.0f * added <= rows) || (tiles < 4 * blocks && 20.0f * added <= rows);
+  return tiles < 4 * blocks && 50.0f * (float)((2 << lg) - 1) < rows;
 }
 
 // LIST: the tets are the hdr->listq_count ones listed at the back of p.tetq.
@@ -441,6 +436,7 @@ __global__ void __launch_bounds__(kSuBlock, SL == kSuSlicesSmall ? 7 : 5) k_slic
             su_share_more((end << lg) / kSuBlock, (long long)gridDim.x, rows, lg)))
       ++lg;
   }
+  
   for (;;) {
     if (threadIdx.x == 0 && su_next_window(sm)) sm.tile = (long long)atomicAdd(&p.hdr->tile_counter, 1ull);
     __syncthreads();
@@ -451,8 +447,9 @@ __global__ void __launch_bounds__(kSuBlock, SL == kSuSlicesSmall ? 7 : 5) k_slic
   flush_counters(p.hdr, ctr);
 }
 
-// The tiles of every job of a batch, claimed from one counter; a tile's job is found in the
-// per-job tile offsets by one warp.  A job's device-detected errors also go to its status word.
+// The tiles of every job of a batch, claimed from one counter bh->chunk at a time; a claim's job is
+// found in the per-job tile offsets by one warp.  A job's device-detected errors also go to its
+// status word.
 template <bool STRICT, bool CULL>
 __global__ void __launch_bounds__(kSuBlock, 7) k_slices_batched(BatchHeader *bh, const JobDesc *jobs,
                                                                const unsigned long long *tile_base, int *status) {
@@ -463,27 +460,41 @@ __global__ void __launch_bounds__(kSuBlock, 7) k_slices_batched(BatchHeader *bh,
   SuSmem<SL> &sm = *reinterpret_cast<SuSmem<SL> *>(su_dyn_smem);
   __shared__ Params sp;
   __shared__ int job_s;
+  // the current tile, the claim's end, and the current job's first tile and the one after its last
+  __shared__ unsigned long long at, claim_end, job_first, job_end;
   const int tid = threadIdx.x;
   TileCounters ctr;
   su_begin(sm);
   const int n = bh->n_jobs;
-  const unsigned long long total = bh->total_tiles;
+  const unsigned long long total = bh->total_tiles, chunk = bh->chunk;
   int cur = -1;
+  if (tid == 0) {
+    at = claim_end = job_first = job_end = 0;
+    job_s = -1;
+  }
   for (;;) {
     if (tid < 32) {
       unsigned long long tile = 0;
-      int claim = 0;
-      if (tid == 0) {
-        claim = su_next_window(sm);
-        if (claim) tile = atomicAdd(&bh->tile_counter, 1ull);
+      int search = 0;
+      if (tid == 0 && su_next_window(sm)) {
+        if (++at >= claim_end) {
+          at = atomicAdd(&bh->tile_counter, chunk);
+          claim_end = at + chunk;
+        }
+        tile = at;
+        if (tile >= total) job_s = -1;
+        else search = 1 + (job_s >= 0 && tile < job_end && tile >= job_first);
+        if (search == 2) sm.tile = (long long)(tile - job_first);
       }
-      claim = __shfl_sync(0xFFFFFFFFu, claim, 0);
-      if (claim) {
+      search = __shfl_sync(0xFFFFFFFFu, search, 0);
+      if (search == 1) {
         tile = __shfl_sync(0xFFFFFFFFu, tile, 0);
-        const int j = tile < total ? find_job_warp(tile_base, n, tile) : -1;
+        const int j = find_job_warp(tile_base, n, tile);
         if (tid == 0) {
-          sm.tile = j < 0 ? 0 : (long long)(tile - tile_base[j]);
           job_s = j;
+          job_first = tile_base[j];
+          job_end = tile_base[j + 1];
+          sm.tile = (long long)(tile - job_first);
         }
       }
     }
@@ -537,15 +548,17 @@ size_t slices_smem_bytes(int slices) {
   return slices <= kSuSlicesSmall ? sizeof(SuSmem<kSuSlicesSmall>) : sizeof(SuSmem<kSuSlices>);
 }
 
-int su_group_log2(long long n_tets, int side, int slab, int slices, long long blocks) {
+int su_group_log2(long long n_tets, int side, int ry, int slab, int slices, long long blocks) {
   if (n_tets < 1) return 0;
-  const double w = (double)side / std::cbrt((double)n_tets / 6.0);
-  const double span = w < slab ? w : slab;  // slices a tet spans, about
+  const double cells = std::cbrt((double)n_tets / 6.0);
+  const double w = (double)side / cells, span = w < slab ? w : slab;  // slices a tet spans, about
   int lg = 0;
   while (lg < kSuMaxGroup && (double)(slices << lg) < span) ++lg;
   while (lg < kSuMaxGroup && (double)(1 << lg) < span && ((n_tets << lg) / kSuBlock) * 2 < blocks) ++lg;
-  while (lg < kSuMaxGroup && (double)(1 << lg) < span &&
-         su_share_more((n_tets << lg) / kSuBlock, blocks, (float)(0.5 * w * span), lg))
+  // a guess of the rows, too high for a mesh that fills only part of its grid: it counts for half,
+  // and for up to two tiles a block
+  const float rows = (float)(0.25 * (double)ry / cells * span);
+  while (lg < kSuMaxGroup && (double)(1 << lg) < span && su_share_more(2 * ((n_tets << lg) / kSuBlock), blocks, rows, lg))
     ++lg;
   return lg;
 }
@@ -610,7 +623,7 @@ int launch_slices(const Params &p_in, int variant, int slices, int sms, cudaStre
   long long grid = (long long)sms * occ;
   // a list's length is known on the device only: the kernel shares its tets among more threads
   const int side = 1 << (kLatticeBits - p.sh);
-  p.lg = list ? 0 : su_group_log2(p.n_tets, side, p.z1 - p.z0, slices, grid);
+  p.lg = list ? 0 : su_group_log2(p.n_tets, side, p.ry, p.z1 - p.z0, slices, grid);
   const int per_tile = kSuBlock >> p.lg;
   const long long tiles = list ? grid : (p.n_tets + per_tile - 1) / per_tile;
   if (grid > tiles) grid = tiles;

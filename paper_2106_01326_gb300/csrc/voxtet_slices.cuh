@@ -15,7 +15,7 @@ constexpr int kSuRows = 1024;   // x-rows per slice of a tet's box in one window
 constexpr int kSuMaxGroup = 7;  // log2 of the most threads that share a tet (a whole block)
 
 // log2 of the threads that share a tet in the slice-unit kernel, from the mesh's size and the grid
-// it goes to (side: the lattice's voxels per axis; slab: the slices produced): a tet of a mesh that
+// it goes to (side: the lattice's voxels per axis; ry: rows per slice; slab: the slices produced): a tet of a mesh that
 // fills its grid spans about w = side / cbrt(n_tets / 6) slices.
 //   - As many threads as make one window hold w slices (`slices` a thread).  Measured on GB300, 64
 //     meshes of 1k-1M tets on 64^3-512^3 grids: 1.54 ms with this many threads, 1.94 with a
@@ -27,7 +27,7 @@ constexpr int kSuMaxGroup = 7;  // log2 of the most threads that share a tet (a 
 //   - More if a tile or two per resident block would be uneven (su_share_more).
 //   - Never more than w: they would have no slice to take (4,200 tets at 64^3: 62 us up to 16
 //     threads a tet, 78 with 64).
-int su_group_log2(long long n_tets, int side, int slab, int slices, long long blocks);
+int su_group_log2(long long n_tets, int side, int ry, int slab, int slices, long long blocks);
 
 // Enqueue the slice-unit kernel for p on `stream`: variant = (list << 3) | (strict << 2) |
 // (cull << 1) | clamp; slices = the slices a thread takes per window (kSuSlicesSmall or
