@@ -1269,10 +1269,10 @@ static int run_voxelize(const Workspace &w, long long n_verts, const int32_t *te
     g_launches.fetch_add(1);
     if (cudaGetLastError() != cudaSuccess) return VOXTET_ERR_CUDA;
   }
-  if (o.sync) {
-    if (cudaStreamSynchronize(stream) != cudaSuccess) return VOXTET_ERR_CUDA;
+  if (o.sync) {  // the copy waits in the stream for the kernels; the wait below is for both
     int bits = 0;
-    if (cudaMemcpy(&bits, &w.hdr->status_bits, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+    if (cudaMemcpyAsync(&bits, &w.hdr->status_bits, sizeof(int), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+        cudaStreamSynchronize(stream) != cudaSuccess)
       return VOXTET_ERR_CUDA;
     return map_status_bits(bits);
   }
@@ -1621,10 +1621,11 @@ static size_t job_slice_bytes(const voxtet_job &j, bool valid) {
   return valid ? align256(voxtet_workspace_size(j.n_tets, j.n_verts, j.res)) : align256(sizeof(Header));
 }
 
-// Builds the host image of the table part of a batch workspace.  Returns the bytes
-// of workspace the batch needs (0 on a batch-level argument error).
+// Builds the host image of the table part of a batch workspace in img (batch_layout(cap).o_slices
+// bytes; nullptr, or a workspace of ws_bytes that is too small: nothing is built).  Returns the bytes of workspace the batch needs (0 on a batch-level
+// argument error).
 static size_t build_batch_image(const voxtet_job *jobs, int n, int cap, const voxtet_opts &o, long long blocks,
-                                char *ws_dev, std::vector<char> *image, int *host_status) {
+                                char *ws_dev, size_t ws_bytes, char *img, int *host_status) {
   const BatchLayout L = batch_layout(cap);
   size_t need = L.o_slices;
   std::vector<int> ok(n);
@@ -1635,9 +1636,8 @@ static size_t build_batch_image(const voxtet_job *jobs, int n, int cap, const vo
     if (host_status) host_status[j] = st;
     need += job_slice_bytes(jobs[j], ok[j]);
   }
-  if (!image) return need;
-  image->assign(L.o_slices, 0);
-  char *img = image->data();
+  if (!img || need > ws_bytes) return need;
+  std::memset(img, 0, L.o_slices);
   BatchHeader *bh = reinterpret_cast<BatchHeader *>(img);
   JobDesc *tab = reinterpret_cast<JobDesc *>(img + L.o_table);
   unsigned long long *tiles = reinterpret_cast<unsigned long long *>(img + L.o_tiles);
@@ -1771,7 +1771,7 @@ size_t voxtet_batch_workspace_size(const voxtet_job *jobs, int32_t n_jobs, int32
   voxtet_opts o;
   voxtet_default_opts(&o);
   std::vector<int> st((size_t)(n_jobs > 0 ? n_jobs : 1));
-  return build_batch_image(jobs, n_jobs, max_jobs > 0 ? max_jobs : 1, o, 0, nullptr, nullptr, st.data());
+  return build_batch_image(jobs, n_jobs, max_jobs > 0 ? max_jobs : 1, o, 0, nullptr, 0, nullptr, st.data());
 }
 
 int voxelize_tets_batched(const voxtet_job *jobs, int32_t n_jobs, void *d_ws, size_t ws_bytes,
@@ -1784,10 +1784,11 @@ int voxelize_tets_batched(const voxtet_job *jobs, int32_t n_jobs, void *d_ws, si
   if (!d_ws || (reinterpret_cast<uintptr_t>(d_ws) & 255)) return VOXTET_ERR_WORKSPACE;
   const int cap = n_jobs > 0 ? n_jobs : 1;
   std::vector<int> hs((size_t)cap, VOXTET_OK);
-  std::vector<char> image;
+  std::vector<char> image(batch_layout(cap).o_slices);
   const long long blocks = batch_blocks(o);
   if (blocks < 1) return VOXTET_ERR_CUDA;
-  const size_t need = build_batch_image(jobs, n_jobs, cap, o, blocks, reinterpret_cast<char *>(d_ws), &image, hs.data());
+  const size_t need =
+      build_batch_image(jobs, n_jobs, cap, o, blocks, reinterpret_cast<char *>(d_ws), ws_bytes, image.data(), hs.data());
   if (need > ws_bytes) return VOXTET_ERR_WORKSPACE;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
   if (cudaMemcpyAsync(d_ws, image.data(), image.size(), cudaMemcpyHostToDevice, stream) != cudaSuccess)
@@ -1834,14 +1835,14 @@ int voxtet_plan_run(voxtet_plan *p, const voxtet_job *jobs, int32_t n_jobs, void
   if (!p || n_jobs < 0 || n_jobs > p->cap || (n_jobs > 0 && !jobs)) return VOXTET_ERR_ARG;
   if (p->in_flight && cudaEventSynchronize(p->done) != cudaSuccess) return VOXTET_ERR_CUDA;
   p->in_flight = false;
-  p->host_status.assign((size_t)(n_jobs > 0 ? n_jobs : 1), VOXTET_OK);
-  std::vector<char> image;
   const long long blocks = batch_blocks(p->opts);
   if (blocks < 1) return VOXTET_ERR_CUDA;
+  // nothing of this plan is in flight, so the pinned image is free
+  std::vector<int> hs((size_t)(n_jobs > 0 ? n_jobs : 1), VOXTET_OK);
   const size_t need =
-      build_batch_image(jobs, n_jobs, p->cap, p->opts, blocks, p->ws, &image, p->host_status.data());
+      build_batch_image(jobs, n_jobs, p->cap, p->opts, blocks, p->ws, p->ws_bytes, p->pinned, hs.data());
   if (need > p->ws_bytes) return VOXTET_ERR_NOMEM;
-  std::memcpy(p->pinned, image.data(), p->image_bytes);
+  p->host_status.swap(hs);
   cudaGraphExec_t &exec = p->exec;
   if (!exec) {  // capture the upload and the kernels once; later runs replay them
     cudaGraph_t g = nullptr;
@@ -1849,6 +1850,10 @@ int voxtet_plan_run(voxtet_plan *p, const voxtet_job *jobs, int32_t n_jobs, void
     cudaMemcpyAsync(p->ws, p->pinned, p->image_bytes, cudaMemcpyHostToDevice, p->cap_stream);
     const unsigned long long before = g_launches.load();
     const int st = launch_batch(p->ws, p->cap, p->opts.mode == 1, p->opts.row_cull != 2, p->cap_stream);
+    // the jobs' status words come back into the image with the batch
+    const size_t o_status = batch_layout(p->cap).o_status;
+    cudaMemcpyAsync(p->pinned + o_status, p->ws + o_status, (size_t)p->cap * sizeof(int), cudaMemcpyDeviceToHost,
+                    p->cap_stream);
     g_launches.store(before);  // captured, not launched
     if (cudaStreamEndCapture(p->cap_stream, &g) != cudaSuccess || st != VOXTET_OK) {
       if (g) cudaGraphDestroy(g);
@@ -1875,9 +1880,9 @@ int voxtet_plan_wait(voxtet_plan *p, int32_t *job_status) {
   if (p->in_flight && cudaEventSynchronize(p->done) != cudaSuccess) return VOXTET_ERR_CUDA;
   p->in_flight = false;
   if (!job_status || p->n_jobs == 0) return VOXTET_OK;
-  const int st = read_job_status(p->ws, p->cap, p->n_jobs, p->host_status.data(), nullptr);
-  if (st != VOXTET_OK) return st;
-  for (int j = 0; j < p->n_jobs; ++j) job_status[j] = p->host_status[j];
+  const int *bits = reinterpret_cast<const int *>(p->pinned + batch_layout(p->cap).o_status);
+  for (int j = 0; j < p->n_jobs; ++j)
+    job_status[j] = p->host_status[j] == VOXTET_OK ? map_status_bits(bits[j]) : p->host_status[j];
   return VOXTET_OK;
 }
 
