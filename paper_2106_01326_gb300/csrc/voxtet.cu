@@ -37,9 +37,8 @@
 //                than 2^20 lattice units go to the tet queue, uncertain rows to
 //                the row queue (tets whose rows overflow it are flagged in the
 //                redo bitmap).
-//   k_exact_rows solves the queued rows with exact integers and ORs them in;
-//   k_exact      the queued whole tets and the redo bitmap's (OR is idempotent,
-//                so redoing a row is harmless).
+//   k_exact      solves the queued rows, the queued whole tets and the redo bitmap's
+//                with exact integers (OR is idempotent, so redoing a row is harmless).
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -59,7 +58,6 @@ namespace voxtet {
 
 __global__ void k_prologue(Header *hdr, uint32_t *redo, long long redo_words, uint32_t *out, long long n_words,
                            int clear) {
-  chain_wait();     // a slab's: the previous slab's bricks are written and cleared
   chain_release();  // the next kernel may be scheduled now; it waits for this one to complete
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -768,19 +766,15 @@ __device__ __forceinline__ void exact_redo(const Params &p, unsigned bi, unsigne
     if ((p.redo[t >> 5] >> (t & 31)) & 1u) exact_tet<STRICT>(p, t);
 }
 
-// The queued rows, in a kernel of their own: the 64-bit row solve needs far fewer registers
-// than the tet path's 128-bit one, so many more threads are resident.
-template <bool STRICT>
-__global__ void __launch_bounds__(128) k_exact_rows(Params p) {
-  chain_wait();  // every row is queued
-  chain_release();
-  const unsigned n_rq = min(p.hdr->rowq_count, p.q_cap), stride = gridDim.x * blockDim.x;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n_rq; i += stride) exact_queued_row<STRICT>(p, p.rowq[i]);
-}
-
+// The queued rows (a thread each), the queued tets (a block each) and, after a row-queue overflow,
+// the flagged ones.  One kernel for all: the 128-bit tet path's registers leave three blocks per SM,
+// 58,368 threads, more than there are queued rows at most sizes (2.3k at 512^3, 20k at 1024^3 for the
+// sliver mesh), and a launch of its own for the rows cost a call 3-4 us.
 template <bool STRICT>
 __global__ void __launch_bounds__(128) k_exact(Params p) {
-  chain_wait();  // every tet is queued
+  // no early release of the next kernel: the brick count's blocks, placed unevenly while these run,
+  // took 15 us longer per slab
+  chain_wait();  // every row and tet is queued
   if (p.vflags) {  // the vertices' error bits, left in verts4[i].w by the fused prologue and snap
     int err = 0;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -789,6 +783,8 @@ __global__ void __launch_bounds__(128) k_exact(Params p) {
     err = __reduce_or_sync(0xFFFFFFFFu, err);
     if ((threadIdx.x & 31) == 0 && err) atomicOr(&p.hdr->status_bits, err);
   }
+  const unsigned n_rq = min(p.hdr->rowq_count, p.q_cap), threads = gridDim.x * blockDim.x;
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n_rq; i += threads) exact_queued_row<STRICT>(p, p.rowq[i]);
   const unsigned n_tq = min((unsigned long long)p.hdr->tetq_count, (unsigned long long)p.n_tets);
   for (unsigned q = blockIdx.x; q < n_tq; q += gridDim.x) exact_tet<STRICT>(p, p.tetq[q]);
   if (p.hdr->rowq_count > p.q_cap) exact_redo<STRICT>(p, blockIdx.x, gridDim.x);
@@ -921,15 +917,14 @@ __device__ __forceinline__ int queue_job(const u64 *pre, int m, u64 x) {
   return a;
 }
 
-// The queued rows of every job as one list, a thread each: which job's rows need it is known only
-// now (a job of wide tets on a fine grid queues many times the rows of one with as many small
-// tets), so the list is spread over all blocks rather than a share of the blocks given to a job
-// beforehand.
+// The exact work of every job: its queued rows (a thread each), its queued tets (a block each) and
+// the redo bitmaps of jobs whose row queue overflowed.  The queues of all jobs make one list each,
+// spread over all blocks: which jobs' rows need exact work is known only now (a job of wide tets on
+// a fine grid queues many times the rows of one with as many small tets).
 template <bool STRICT>
-__global__ void __launch_bounds__(128) k_exact_rows_batched(const BatchHeader *bh, const JobDesc *jobs) {
+__global__ void __launch_bounds__(128) k_exact_batched(const BatchHeader *bh, const JobDesc *jobs) {
   __shared__ u64 pre[kQueueJobs + 1];
-  chain_wait();  // every row is queued
-  chain_release();
+  chain_wait();  // every row and tet is queued
   const int n = bh->n_jobs;
   for (int j0 = 0; j0 < n; j0 += kQueueJobs) {
     const int m = min(kQueueJobs, n - j0);
@@ -937,25 +932,12 @@ __global__ void __launch_bounds__(128) k_exact_rows_batched(const BatchHeader *b
       const Params &p = jobs[j0 + j].p;
       return min(p.hdr->rowq_count, p.q_cap);
     });
-    const u64 total = pre[m];
-    const unsigned stride = gridDim.x * blockDim.x;
-    for (u64 i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+    const unsigned threads = gridDim.x * blockDim.x;
+    for (u64 i = blockIdx.x * blockDim.x + threadIdx.x; i < pre[m]; i += threads) {
       const int j = queue_job(pre, m, i);
       const Params &p = jobs[j0 + j].p;
       exact_queued_row<STRICT>(p, p.rowq[i - pre[j]]);
     }
-  }
-}
-
-// The queued tets of every job, a block each, and the redo bitmaps of jobs whose row queue
-// overflowed.
-template <bool STRICT>
-__global__ void __launch_bounds__(128) k_exact_batched(const BatchHeader *bh, const JobDesc *jobs) {
-  __shared__ u64 pre[kQueueJobs + 1];
-  chain_wait();  // every tet is queued
-  const int n = bh->n_jobs;
-  for (int j0 = 0; j0 < n; j0 += kQueueJobs) {
-    const int m = min(kQueueJobs, n - j0);
     queue_prefix(pre, m, [&](int j) {
       const Params &p = jobs[j0 + j].p;
       return (unsigned)min((long long)p.hdr->tetq_count, p.n_tets);
@@ -1002,8 +984,7 @@ static VoxKernel voxelize_kernel(int idx) {
 struct DeviceInfo {
   int sms = 0;
   int occ[kVariants] = {};  // resident blocks per SM of each k_voxelize variant
-  int occ_exact = 0;        // resident blocks per SM of the exact kernels (tets, rows)
-  int occ_rows = 0;
+  int occ_exact = 0;        // resident blocks per SM of the exact kernel
   bool ready = false;
 };
 static DeviceInfo g_dev[kMaxDevices];
@@ -1055,9 +1036,7 @@ static cudaError_t device_info(DeviceInfo *&out) {
                                                             kSliceTableBytesMax);
       }
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.occ_exact, k_exact<false>, kExactBlock, 0);
-      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.occ_rows, k_exact_rows<false>, kExactBlock, 0);
       if (e == cudaSuccess && d.occ_exact < 1) d.occ_exact = 1;
-      if (e == cudaSuccess && d.occ_rows < 1) d.occ_rows = 1;
       if (e == cudaSuccess) d.ready = true;
     }
     g_dev_lock.store(0);
@@ -1257,12 +1236,7 @@ static int run_voxelize(const Workspace &w, long long n_verts, const int32_t *te
       if (cudaEventRecord(t_prof.stop, stream) != cudaSuccess) return VOXTET_ERR_CUDA;
       t_prof.pending = true;
     }
-    // one wave of resident blocks each: the queued rows are spread evenly over the threads
-    const unsigned rg = (unsigned)dev->sms * (unsigned)dev->occ_rows;
-    if (launch_chained(o.mode == 1 ? k_exact_rows<true> : k_exact_rows<false>, rg, kExactBlock, 0, stream, p) !=
-        cudaSuccess)
-      return VOXTET_ERR_CUDA;
-    g_launches.fetch_add(1);
+    // one wave of resident blocks: the queued rows are spread evenly over the threads
     const unsigned eg = (unsigned)dev->sms * (unsigned)dev->occ_exact;
     if (launch_chained(o.mode == 1 ? k_exact<true> : k_exact<false>, eg, kExactBlock, 0, stream, p) != cudaSuccess)
       return VOXTET_ERR_CUDA;
@@ -1279,22 +1253,14 @@ static int run_voxelize(const Workspace &w, long long n_verts, const int32_t *te
   return VOXTET_OK;
 }
 
-// chained: after a launch of this library in the same call (see launch_chained).
-static int launch_prologue(const Workspace &w, uint32_t *out, long long n_words, int clear, cudaStream_t stream,
-                           bool chained = false) {
+static int launch_prologue(const Workspace &w, uint32_t *out, long long n_words, int clear, cudaStream_t stream) {
   DeviceInfo *dev = nullptr;
   if (device_info(dev) != cudaSuccess) return VOXTET_ERR_CUDA;
   long long blocks = clear ? (n_words / 4 + 255) / 256 : (w.redo_words + 255) / 256;
   const long long cap = (long long)dev->sms * 8;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
-  if (chained) {
-    if (launch_chained(k_prologue, (unsigned)blocks, 256, 0, stream, w.hdr, w.redo, w.redo_words, out, n_words,
-                       clear) != cudaSuccess)
-      return VOXTET_ERR_CUDA;
-  } else {
-    k_prologue<<<(unsigned)blocks, 256, 0, stream>>>(w.hdr, w.redo, w.redo_words, out, n_words, clear);
-  }
+  k_prologue<<<(unsigned)blocks, 256, 0, stream>>>(w.hdr, w.redo, w.redo_words, out, n_words, clear);
   g_launches.fetch_add(1);
   return cudaGetLastError() == cudaSuccess ? VOXTET_OK : VOXTET_ERR_CUDA;
 }
@@ -1708,7 +1674,7 @@ static long long batch_blocks(const voxtet_opts &o) {
   return (long long)dev->sms * slices_batched_blocks(o.mode == 1, o.row_cull != 2);
 }
 
-constexpr int kBatchLaunches = 4;
+constexpr int kBatchLaunches = 3;
 
 // Enqueues the batch kernels on `stream` (the table must already be uploaded); `cull`: the
 // batch's jobs skip rows outside each slice's cross-section (opts->row_cull != 2).
@@ -1724,9 +1690,6 @@ static int launch_batch(char *ws, int cap, bool strict, bool cull, cudaStream_t 
   k_prep_batched<<<(unsigned)dev->sms * 8, kPrepBlock, 0, stream>>>(bh, tab, prep, status);
   if (cudaGetLastError() != cudaSuccess) return VOXTET_ERR_CUDA;
   if (launch_slices_batched(bh, tab, tiles, status, strict, cull, dev->sms, stream) != VOXTET_OK) return VOXTET_ERR_CUDA;
-  if (launch_chained(strict ? k_exact_rows_batched<true> : k_exact_rows_batched<false>,
-                     (unsigned)dev->sms * (unsigned)dev->occ_rows, kExactBlock, 0, stream, bh, tab) != cudaSuccess)
-    return VOXTET_ERR_CUDA;
   if (launch_chained(strict ? k_exact_batched<true> : k_exact_batched<false>,
                      (unsigned)dev->sms * (unsigned)dev->occ_exact, kExactBlock, 0, stream, bh, tab) != cudaSuccess)
     return VOXTET_ERR_CUDA;
@@ -2097,7 +2060,8 @@ __global__ void __launch_bounds__(kCompactBlock) k_brick_count4(SlabBricks s, un
 // thread: a slab of the default size has 4096 blocks, one turn of the loop (a count a thread, four
 // turns: 6.6 us).
 __global__ void __launch_bounds__(1024) k_brick_scan(unsigned long long *counts, long long n_blocks,
-                                                     SparseHeader *sh, const Header *slab_hdr) {
+                                                     SparseHeader *sh, Header *slab_hdr, uint32_t *redo,
+                                                     long long redo_words) {
   __shared__ unsigned long long warp_sums[32];
   __shared__ unsigned long long carry;
   chain_wait();  // every brick is counted
@@ -2108,6 +2072,10 @@ __global__ void __launch_bounds__(1024) k_brick_scan(unsigned long long *counts,
     sh->sticky_bits |= slab_hdr->status_bits;
   }
   __syncthreads();
+  if (redo) {  // another slab follows: its launches find the header and the bitmap zeroed
+    if (tid < (int)(sizeof(Header) / 4)) reinterpret_cast<uint32_t *>(slab_hdr)[tid] = 0u;
+    for (long long i = tid; i < redo_words; i += 1024) redo[i] = 0u;
+  }
   for (long long base = 0; base < n_blocks; base += 4096) {
     const long long i = base + 4 * tid;
     unsigned long long v[4], mine = 0;
@@ -2357,10 +2325,8 @@ int voxelize_tets_sparse(const float *d_verts, int64_t n_verts, const int32_t *d
     GridDims gs = g;
     gs.z0 = z0;
     gs.z1 = z0 + slab_depth < g.rz ? z0 + slab_depth : g.rz;
-    if (si > 0) {  // the slab is zero: the previous slab's k_brick_write cleared every brick it held
-      st = launch_prologue(w, dense, gs.out_words(), 0, stream, true);
-      if (st != VOXTET_OK) return st;
-    }
+    // from the second slab on, the slab is zero (the previous slab's k_brick_write cleared every
+    // brick it held) and so are the header and the redo bitmap (its k_brick_scan)
     st = run_voxelize(w, n_verts, d_tets, n_tets, gs, dense, inner, stream);
     if (st != VOXTET_OK) return st;
     SlabBricks s;
@@ -2381,7 +2347,11 @@ int voxelize_tets_sparse(const float *d_verts, int64_t n_verts, const int32_t *d
     } else {
       e = launch_chained(k_brick_count, (unsigned)nb, kCompactBlock, 0, stream, s, block_counts, masks);
     }
-    if (e == cudaSuccess) e = launch_chained(k_brick_scan, 1u, 1024u, 0, stream, block_counts, nb, sh, w.hdr);
+    bool last = true;
+    for (int sn = si + 1; sn < n_slabs; ++sn) last = last && !((marks[(size_t)sn >> 5] >> (sn & 31)) & 1u);
+    if (e == cudaSuccess)
+      e = launch_chained(k_brick_scan, 1u, 1024u, 0, stream, block_counts, nb, sh, w.hdr, last ? nullptr : w.redo,
+                         w.redo_words);
     if (e == cudaSuccess)
       e = launch_chained(k_brick_write, (unsigned)nb, kCompactBlock, 0, stream, s, block_counts, masks, d_brick_keys,
                          d_brick_words, (long long)max_bricks);
