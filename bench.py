@@ -743,8 +743,7 @@ def run_ours(args):
     peak, peak_kind = load_peaks()
     achieved = alg_bytes / (kmean / 1000.0) / 1e9
     # the launches the library's profile events bracket
-    main_kernel = ("k_slices + k_voxelize (list pass over the tets the slice-unit kernel leaves)"
-                   if kernel == 2 else "k_voxelize")
+    main_kernel = "k_slices" if kernel == 2 else "k_voxelize"
     traffic_kernel = "k_slices" if kernel == 2 else "k_voxelize"
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,

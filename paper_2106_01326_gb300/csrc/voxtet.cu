@@ -1217,11 +1217,10 @@ static int run_voxelize(const Workspace &w, long long n_verts, const int32_t *te
           return VOXTET_ERR_CUDA;
         g_launches.fetch_add(1);
       }
-      // slice units for the tets that fit them, then the span kernel over the tets it listed
-      // 16 slices per tet (7 blocks per SM) up to 512 voxels per side, where a tet of a mesh
-      // fine enough for the grid spans a few slices (sliver mesh: at most 13), 32 above
-      // (measured on GB300, sliver mesh 512^3: 308 -> 285 us with 16); a tet spanning more
-      // goes to the list pass either way
+      // 16 slices a thread and window (7 blocks per SM) up to 512 voxels per side, where a tet of a
+      // mesh fine enough for the grid spans a few slices (sliver mesh: at most 13), 32 above
+      // (measured on GB300, sliver mesh 512^3: 308 -> 285 us with 16; a 4096^3 torus in slabs 4.19 ms
+      // with 32, 4.28 with 16)
       const int cap = g.longest() <= 512 ? kSuSlicesSmall : kSuSlices;
       if (launch_slices(p, variant, cap, dev->sms, stream) != VOXTET_OK) return VOXTET_ERR_CUDA;
       g_launches.fetch_add(1);
