@@ -1222,7 +1222,7 @@ static int run_voxelize(const Workspace &w, long long n_verts, const int32_t *te
       // (measured on GB300, sliver mesh 512^3: 308 -> 285 us with 16; a 4096^3 torus in slabs 4.19 ms
       // with 32, 4.28 with 16)
       const int cap = g.longest() <= 512 ? kSuSlicesSmall : kSuSlices;
-      if (launch_slices(p, variant, cap, dev->sms, stream) != VOXTET_OK) return VOXTET_ERR_CUDA;
+      if (launch_slices(p, variant >> 1, cap, dev->sms, stream) != VOXTET_OK) return VOXTET_ERR_CUDA;
       g_launches.fetch_add(1);
     } else {
       if (launch_chained(voxelize_kernel(variant), (unsigned)grid, kBlock, slice_table_bytes(p.max_slices), stream,

@@ -276,7 +276,7 @@ __device__ __forceinline__ long long su_tet(const Params &p, long long i, long l
 }
 
 // Phase (3): rows b0 .. b0 + n - 1 of slice k of the tet in `slot` (place t of the launch).
-template <bool STRICT, bool CLAMP, bool LIST, bool BATCH, int SL>
+template <bool STRICT, bool PAIRS, bool LIST, bool BATCH, int SL>
 __device__ __forceinline__ void su_walk(const Params &p, SuSmem<SL> &sm, int slot, long long t, int k, int b0, int n) {
   const float4 *R = reinterpret_cast<const float4 *>(sm.rec + slot * kSuRec);
   const float4 qa = R[0], qb = R[1], qg = R[2], qi = R[3];
@@ -315,13 +315,14 @@ __device__ __forceinline__ void su_walk(const Params &p, SuSmem<SL> &sm, int slo
     do {
       uint32_t lo, hi;
       bool live;
-      bool a = row_bounds<STRICT, CLAMP>(f, bf, lo, hi, live);
+      bool a = row_bounds<STRICT>(f, bf, lo, hi, live);
       if (a) {
         a = row_refine<STRICT>(f, R[kRecE / 4], up1, up2, bf);
         live = !a && __uint_as_float(lo) <= __uint_as_float(hi);
       }
       amb = amb + amb + (a ? 1u : 0u);  // the last row in the lowest bit
-      row_or<BATCH>(row, off, lo, hi, live);
+      if (PAIRS) row_or_pairs(row, off, lo, hi, live);
+      else row_or<BATCH>(row, off, lo, hi, live);
       bf += 1.f;
       off += (uint32_t)p.W;
     } while (bf != b_end);
@@ -339,7 +340,7 @@ __device__ __forceinline__ void su_walk(const Params &p, SuSmem<SL> &sm, int slo
 // loop claims a tile or moves to the tile's next window: a loop of its own around these phases
 // cost the row loop its reconvergence (measured on GB300, sliver mesh at 512^3: 26.7 -> 15.9
 // active lanes, 262 -> 440 us).
-template <bool STRICT, bool CULL, bool CLAMP, bool TALL, bool LIST, bool BATCH, int SL>
+template <bool STRICT, bool CULL, bool PAIRS, bool TALL, bool LIST, bool BATCH, int SL>
 __device__ __forceinline__ void su_pass(const Params &p, long long base, long long end, int lg, SuSmem<SL> &sm,
                                         TileCounters &ctr) {
   const int tid = threadIdx.x;
@@ -385,7 +386,7 @@ __device__ __forceinline__ void su_pass(const Params &p, long long base, long lo
     const int k = c0 + ((int)((u >> 7) & 31u) << lg) + (slot & ((1 << lg) - 1));
     const int b0 = (int)((u >> 12) & 1023u) + r0, n = (int)(u >> 22) + 1;
     ctr.rows += (unsigned)n;
-    su_walk<STRICT, CLAMP, LIST, BATCH, SL>(p, sm, slot, base + (slot >> lg), k, b0, n);
+    su_walk<STRICT, PAIRS, LIST, BATCH, SL>(p, sm, slot, base + (slot >> lg), k, b0, n);
   }
   flush_stage(p, sm.stage);
 }
@@ -418,8 +419,9 @@ static __host__ __device__ __forceinline__ bool su_share_more(long long tiles, l
   return tiles < 4 * blocks && 50.0f * (float)((2 << lg) - 1) < rows;
 }
 
-// LIST: the tets are the hdr->listq_count ones listed at the back of p.tetq.
-template <bool STRICT, bool CULL, bool CLAMP, bool LIST, int SL>
+// LIST: the tets are the hdr->listq_count ones listed at the back of p.tetq.  PAIRS: rows are ORed in
+// pairs of words.
+template <bool STRICT, bool CULL, bool PAIRS, bool LIST, int SL>
 __global__ void __launch_bounds__(kSuBlock, SL == kSuSlicesSmall ? 7 : 5) k_slices(Params p) {
   chain_wait();  // vertices snapped, header zeroed, tets listed
   chain_release();
@@ -442,7 +444,7 @@ __global__ void __launch_bounds__(kSuBlock, SL == kSuSlicesSmall ? 7 : 5) k_slic
     __syncthreads();
     const long long base = sm.tile * (kSuBlock >> lg);
     if (base >= end) break;
-    su_pass<STRICT, CULL, CLAMP, SL == kSuSlices, LIST, false, SL>(p, base, end, lg, sm, ctr);
+    su_pass<STRICT, CULL, PAIRS, SL == kSuSlices, LIST, false, SL>(p, base, end, lg, sm, ctr);
   }
   flush_counters(p.hdr, ctr);
 }
@@ -518,30 +520,23 @@ __global__ void __launch_bounds__(kSuBlock, 7) k_slices_batched(BatchHeader *bh,
 
 typedef void (*SuKernel)(Params);
 
-template <int SL>
+// Variant (list << 2) | (strict << 1) | cull.
+template <bool PAIRS, int SL>
 static SuKernel su_kernel(int v) {
   switch (v) {
-    case 0: return k_slices<false, false, false, false, SL>;
-    case 1: return k_slices<false, false, true, false, SL>;
-    case 2: return k_slices<false, true, false, false, SL>;
-    case 3: return k_slices<false, true, true, false, SL>;
-    case 4: return k_slices<true, false, false, false, SL>;
-    case 5: return k_slices<true, false, true, false, SL>;
-    case 6: return k_slices<true, true, false, false, SL>;
-    case 7: return k_slices<true, true, true, false, SL>;
-    case 8: return k_slices<false, false, false, true, SL>;
-    case 9: return k_slices<false, false, true, true, SL>;
-    case 10: return k_slices<false, true, false, true, SL>;
-    case 11: return k_slices<false, true, true, true, SL>;
-    case 12: return k_slices<true, false, false, true, SL>;
-    case 13: return k_slices<true, false, true, true, SL>;
-    case 14: return k_slices<true, true, false, true, SL>;
-    default: return k_slices<true, true, true, true, SL>;
+    case 0: return k_slices<false, false, PAIRS, false, SL>;
+    case 1: return k_slices<false, true, PAIRS, false, SL>;
+    case 2: return k_slices<true, false, PAIRS, false, SL>;
+    case 3: return k_slices<true, true, PAIRS, false, SL>;
+    case 4: return k_slices<false, false, PAIRS, true, SL>;
+    case 5: return k_slices<false, true, PAIRS, true, SL>;
+    case 6: return k_slices<true, false, PAIRS, true, SL>;
+    default: return k_slices<true, true, PAIRS, true, SL>;
   }
 }
 
 constexpr int kSuMaxDevices = 64;
-static int g_su_occ[kSuMaxDevices][2][16];  // resident blocks per SM per capacity and variant, 0 = not yet queried
+static int g_su_occ[kSuMaxDevices][3][8];  // resident blocks per SM per form and variant, 0 = not yet queried
 static std::atomic<int> g_su_lock{0};
 
 size_t slices_smem_bytes(int slices) {
@@ -603,10 +598,16 @@ int launch_slices_batched(BatchHeader *bh, const JobDesc *jobs, const unsigned l
 int launch_slices(const Params &p_in, int variant, int slices, int sms, cudaStream_t stream) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kSuMaxDevices) return VOXTET_ERR_CUDA;
-  const int c = slices <= kSuSlicesSmall ? 0 : 1;
-  SuKernel kern = c == 0 ? su_kernel<kSuSlicesSmall>(variant & 15) : su_kernel<kSuSlices>(variant & 15);
+  // Pairs of words where the ORs are the bound (32-slice windows: grids above 512 per side) and every
+  // row starts on an 8-byte boundary.  Measured on GB300: sliver mesh at 1024^3 1018 -> 996 us,
+  // 162,000 tets at 1024^3 656 -> 606, 1.3 M at 2048^3 4.77 -> 4.40 ms, 4096^3 torus in slabs 4.22 ->
+  // 3.89 ms; at 512^3, bound by issue, the longer masks cost more than they save.
+  const int c = slices <= kSuSlicesSmall ? 0 : (p_in.W & 1) != 0 || (reinterpret_cast<uintptr_t>(p_in.out) & 7) != 0 ? 1 : 2;
+  const SuKernel kern = c == 0   ? su_kernel<false, kSuSlicesSmall>(variant & 7)
+                        : c == 1 ? su_kernel<false, kSuSlices>(variant & 7)
+                                 : su_kernel<true, kSuSlices>(variant & 7);
   const size_t smem = slices_smem_bytes(slices);
-  int occ = g_su_occ[dev][c][variant & 15];
+  int occ = g_su_occ[dev][c][variant & 7];
   if (occ == 0) {
     while (g_su_lock.exchange(1)) {
     }
@@ -614,12 +615,12 @@ int launch_slices(const Params &p_in, int variant, int slices, int sms, cudaStre
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kSuBlock, smem);
     if (e == cudaSuccess && occ < 1) occ = 1;
-    if (e == cudaSuccess) g_su_occ[dev][c][variant & 15] = occ;
+    if (e == cudaSuccess) g_su_occ[dev][c][variant & 7] = occ;
     g_su_lock.store(0);
     if (e != cudaSuccess) return VOXTET_ERR_CUDA;
   }
   Params p = p_in;
-  const bool list = (variant & 8) != 0;
+  const bool list = (variant & 4) != 0;
   long long grid = (long long)sms * occ;
   // a list's length is known on the device only: the kernel shares its tets among more threads
   const int side = 1 << (kLatticeBits - p.sh);

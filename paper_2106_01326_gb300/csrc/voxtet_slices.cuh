@@ -29,9 +29,9 @@ constexpr int kSuMaxGroup = 7;  // log2 of the most threads that share a tet (a 
 //     threads a tet, 78 with 64).
 int su_group_log2(long long n_tets, int side, int ry, int slab, int slices, long long blocks);
 
-// Enqueue the slice-unit kernel for p on `stream`: variant = (list << 3) | (strict << 2) |
-// (cull << 1) | clamp; slices = the slices a thread takes per window (kSuSlicesSmall or
-// kSuSlices); list = the tets are those k_slab_list listed.  Returns VOXTET_OK or VOXTET_ERR_CUDA.
+// Enqueue the slice-unit kernel for p on `stream`: variant = (list << 2) | (strict << 1) | cull;
+// slices = the slices a thread takes per window (kSuSlicesSmall or kSuSlices); list = the tets are
+// those k_slab_list listed.  Returns VOXTET_OK or VOXTET_ERR_CUDA.
 int launch_slices(const Params &p, int variant, int slices, int sms, cudaStream_t stream);
 
 // Enqueue the slice-unit kernel over a batch's jobs (tile_base: the jobs' tile offsets, tiles of

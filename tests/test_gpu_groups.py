@@ -138,3 +138,22 @@ def test_batch_of_unlike_jobs(vt):
         for k, (sp, ref) in enumerate(zip(specs, refs)):
             _same(sp.out, ref, k)
     assert int(store[0]) == -1 and int(store[at + vt.grid_words(64)]) == -1
+
+
+@pytest.mark.parametrize("rx,shift", [(640, 0), (640, 1), (608, 0), (609, 0), (1000, 0), (1000, 3), (700, 2)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_rows_in_pairs_of_words(vt, rx, shift, mode):
+    """Grids above 512 per side: rows of even and odd numbers of words in grids that start on 8-byte and
+    on 4-byte boundaries, tets of 1 to 400 columns (rows of one pair, two, and whole pairs between)."""
+    import torch
+
+    dims, h = (rx, 24, 18), 1.0 / 1024
+    verts, tets = _soup(rx, 400, 24, 2, 24, (0.6, 1, 1))
+    verts = verts * np.array([dims[0] * h, dims[1] * h, dims[2] * h], dtype=np.float32)
+    ref = oracle.voxelize_grid(verts, tets, (0, 0, 0), h, dims, mode=mode)
+    v, t = _cuda(verts, tets)
+    w = (rx + 31) // 32
+    store = torch.full((dims[1] * dims[2] * w + 8,), -1, dtype=torch.int32, device="cuda")
+    out = store[shift:shift + dims[1] * dims[2] * w].view(dims[2], dims[1], w)
+    _same(vt.voxelize_grid(v, t, (0, 0, 0), h, dims, out=out, mode=mode), ref, (rx, shift))
+    assert bool((store[:shift] == -1).all()) and bool((store[shift + ref.size:] == -1).all())
