@@ -2118,7 +2118,8 @@ __global__ void __launch_bounds__(1024) k_brick_scan(unsigned long long *counts,
 // word r of brick l: a warp-wide load of row r is one contiguous run), then writes
 // every non-empty brick with two 128-byte stores.
 // Only the bricks the count found non-empty are read again: at 4096^3 in slabs of 64 slices a slab
-// is 128 MiB, about a quarter of it in such bricks.
+// is 128 MiB, about a quarter of it in such bricks.  The output is stored as streaming data, so that
+// the slab, which the next launches use again, keeps its place in L2 (4096^3 torus 3.86 -> 3.72 ms).
 __global__ void __launch_bounds__(kCompactBlock) k_brick_write(SlabBricks s, const unsigned long long *block_offsets,
                                                                const uint4 *masks, uint64_t *keys, uint32_t *words,
                                                                long long cap) {
@@ -2169,8 +2170,8 @@ __global__ void __launch_bounds__(kCompactBlock) k_brick_write(SlabBricks s, con
     mm &= mm - 1;
     if (slot >= (unsigned long long)cap) break;
     uint32_t *dst = words + slot * kBrickWords;
-    dst[lane] = stage[warp][lane][j];
-    dst[32 + lane] = stage[warp][32 + lane][j];
+    __stcs(dst + lane, stage[warp][lane][j]);
+    __stcs(dst + 32 + lane, stage[warp][32 + lane][j]);
   }
 }
 
