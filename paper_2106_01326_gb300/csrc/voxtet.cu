@@ -796,7 +796,7 @@ __global__ void __launch_bounds__(128) k_exact(Params p) {
 // slice-unit kernel's batched form is in voxtet_slices.cu.
 
 constexpr int kPrepBlock = 256;
-constexpr int kZeroWords = 2048;  // words a zeroing chunk covers (8 KB)
+constexpr int kZeroWords = 8192;  // words a zeroing chunk covers (32 KB)
 constexpr int kPrepVerts = 512;   // vertices a snapping chunk covers
 
 // Chunks of job work in the prologue: first its grid's (the first one also zeroes its header and
@@ -813,7 +813,7 @@ static __host__ __device__ unsigned long long prep_chunks(const JobDesc &d) {
 __device__ __forceinline__ void zero_words(uint32_t *w, int n) {
   if ((reinterpret_cast<uintptr_t>(w) & 15) == 0) {
     uint4 *w4 = reinterpret_cast<uint4 *>(w);
-    for (int i = threadIdx.x; i < n / 4; i += kPrepBlock) w4[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = threadIdx.x; i < n / 4; i += kPrepBlock) __stcg(w4 + i, make_uint4(0u, 0u, 0u, 0u));
     for (int i = (n & ~3) + (int)threadIdx.x; i < n; i += kPrepBlock) w[i] = 0u;
   } else {
     for (int i = threadIdx.x; i < n; i += kPrepBlock) w[i] = 0u;
@@ -824,8 +824,9 @@ __device__ __forceinline__ void zero_words(uint32_t *w, int n) {
 // snapped, in one launch: chunk u belongs to the job j with prep_base[j] <= u < prep_base[j + 1].
 // A vertex's error bits go to the job's status word, which the table's upload has zeroed, so
 // nothing here orders against the headers' zeroing.  Bound by its stores: 16-byte stores of whole
-// chunks and one warp-wide job search per chunk (word stores with a search per thread, and a
-// separate snap, took 178 us for 64 jobs of 64^3-512^3 grids, 332 MB).
+// chunks and one warp-wide job search per chunk (64 jobs of 64^3-512^3 grids, 332 MB: 74 us, where
+// word stores with a search per thread and a separate snap took 178; chunks of 32 KB take 14 us off
+// that replay against chunks of 8 KB).
 __global__ void __launch_bounds__(kPrepBlock) k_prep_batched(const BatchHeader *bh, const JobDesc *jobs,
                                                              const unsigned long long *prep_base, int *status) {
   chain_release();
