@@ -824,9 +824,8 @@ __device__ __forceinline__ void zero_words(uint32_t *w, int n) {
 // snapped, in one launch: chunk u belongs to the job j with prep_base[j] <= u < prep_base[j + 1].
 // A vertex's error bits go to the job's status word, which the table's upload has zeroed, so
 // nothing here orders against the headers' zeroing.  Bound by its stores: 16-byte stores of whole
-// chunks and one warp-wide job search per chunk (64 jobs of 64^3-512^3 grids, 332 MB: 74 us, where
-// word stores with a search per thread and a separate snap took 178; chunks of 32 KB take 14 us off
-// that replay against chunks of 8 KB).
+// chunks and one warp-wide job search per chunk (64 jobs of 64^3-512^3 grids, 332 MB: 57 us, 74
+// with chunks of 8 KB; word stores with a search per thread and a separate snap took 178).
 __global__ void __launch_bounds__(kPrepBlock) k_prep_batched(const BatchHeader *bh, const JobDesc *jobs,
                                                              const unsigned long long *prep_base, int *status) {
   chain_release();
@@ -929,9 +928,12 @@ __global__ void __launch_bounds__(128) k_exact_batched(const BatchHeader *bh, co
   const int n = bh->n_jobs;
   for (int j0 = 0; j0 < n; j0 += kQueueJobs) {
     const int m = min(kQueueJobs, n - j0);
+    bool more = false;  // queued tets or an overflown row queue: rare, so looked for along the way
     queue_prefix(pre, m, [&](int j) {
       const Params &p = jobs[j0 + j].p;
-      return min(p.hdr->rowq_count, p.q_cap);
+      const unsigned rows = p.hdr->rowq_count, cap = p.q_cap;
+      more |= p.hdr->tetq_count != 0 || rows > cap;
+      return min(rows, cap);
     });
     const unsigned threads = gridDim.x * blockDim.x;
     for (u64 i = blockIdx.x * blockDim.x + threadIdx.x; i < pre[m]; i += threads) {
@@ -939,6 +941,7 @@ __global__ void __launch_bounds__(128) k_exact_batched(const BatchHeader *bh, co
       const Params &p = jobs[j0 + j].p;
       exact_queued_row<STRICT>(p, p.rowq[i - pre[j]]);
     }
+    if (!__syncthreads_or(more)) continue;
     queue_prefix(pre, m, [&](int j) {
       const Params &p = jobs[j0 + j].p;
       return (unsigned)min((long long)p.hdr->tetq_count, p.n_tets);

@@ -110,7 +110,8 @@ def test_wide_tets_few_rows_left_to_the_exact_kernels(vt, n, res, mode):
     assert st["fallback_rows"] < 0.01 * st["rows"], st
 
 
-def test_batch_of_unlike_jobs(vt):
+@pytest.mark.parametrize("use_filter", [True, False])
+def test_batch_of_unlike_jobs(vt, use_filter):
     """One batch with jobs of one tet, of wide tets, of many small ones, without tets, in lattice
     coordinates and with an unaligned grid; each job's grid and status are its own."""
     import torch
@@ -128,13 +129,19 @@ def test_batch_of_unlike_jobs(vt):
         specs.append(batch.JobSpec(batch.Mesh(v, t), res, store[at:at + w].view(res, res, -1)))
         at += w
         refs.append(oracle.voxelize(verts, tets, (0, 0, 0), 1.0 / res, res) if n else np.zeros((res, res, (res + 31) // 32), np.uint32))
+    # a tet wider than the filter path's integers: the batch's exact kernel takes it
+    wide = np.array([[-0.9, -0.9, -0.5], [1.9, 0.1, 0.4], [0.2, 1.9, 0.6], [0.3, 0.4, 1.7]], dtype=np.float32)
+    v, t = _cuda(wide, np.arange(4, dtype=np.int32).reshape(1, 4))
+    specs.append(batch.JobSpec(batch.Mesh(v, t), 32, store[at:at + vt.grid_words(32)].view(32, 32, -1)))
+    at += vt.grid_words(32)
+    refs.append(oracle.voxelize(wide, np.arange(4, dtype=np.int32).reshape(1, 4), (0, 0, 0), 1.0 / 32, 32))
     bad = _soup(8, 60, 64, 1, 9)
     bad_v = bad[0].copy()
     bad_v[7, 1] = np.nan
     v, t = _cuda(bad_v, bad[1])
     specs.append(batch.JobSpec(batch.Mesh(v, t), 64, store[at:at + vt.grid_words(64)].view(64, 64, -1)))
     for _ in range(2):
-        assert batch.voxelize_batched(specs) == [vt.OK] * len(refs) + [vt.ERR_NAN]
+        assert batch.voxelize_batched(specs, use_filter=use_filter) == [vt.OK] * len(refs) + [vt.ERR_NAN]
         for k, (sp, ref) in enumerate(zip(specs, refs)):
             _same(sp.out, ref, k)
     assert int(store[0]) == -1 and int(store[at + vt.grid_words(64)]) == -1
