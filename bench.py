@@ -79,7 +79,8 @@ def kernel_source_digest() -> str:
     import hashlib
 
     h = hashlib.sha256()
-    for name in ("voxtet.cu", "voxtet_slices.cu", "voxtet_device.cuh", "voxtet_slices.cuh", "tet_math.cuh"):
+    for name in ("voxtet.cu", "voxtet_slices.cu", "voxtet_batch.cuh", "voxtet_device.cuh", "voxtet_rows.cuh",
+                 "voxtet_slices.cuh", "tet_math.cuh"):
         with open(os.path.join(ROOT, "paper_2106_01326_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()
