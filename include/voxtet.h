@@ -276,11 +276,13 @@ typedef struct voxtet_plan voxtet_plan;
 
 int voxtet_plan_create(void *d_workspace, size_t ws_bytes, int32_t max_jobs, const voxtet_opts *opts,
                        voxtet_plan **plan);
-/* Enqueue a batch on `stream`; VOXTET_ERR_NOMEM if it does not fit the workspace. */
+/* Enqueue a batch on `stream`; VOXTET_ERR_NOMEM if it does not fit the workspace.  After a run
+ * that failed (other than by VOXTET_ERR_ARG, which changes nothing) the plan has no last run. */
 int voxtet_plan_run(voxtet_plan *plan, const voxtet_job *jobs, int32_t n_jobs, void *stream);
 /* 1 if the plan's last run has finished, 0 if not, negative on error (does not block). */
 int voxtet_plan_query(voxtet_plan *plan);
-/* Wait for the last run; fill job_status (HOST int32[n_jobs], may be NULL). */
+/* Wait for the last run; fill job_status (HOST int32[n_jobs of that run], may be NULL; left as it is
+ * if there is no last run). */
 int voxtet_plan_wait(voxtet_plan *plan, int32_t *job_status);
 void voxtet_plan_destroy(voxtet_plan *plan);
 

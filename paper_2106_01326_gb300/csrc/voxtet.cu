@@ -1801,6 +1801,7 @@ int voxtet_plan_run(voxtet_plan *p, const voxtet_job *jobs, int32_t n_jobs, void
   if (!p || n_jobs < 0 || n_jobs > p->cap || (n_jobs > 0 && !jobs)) return VOXTET_ERR_ARG;
   if (p->in_flight && cudaEventSynchronize(p->done) != cudaSuccess) return VOXTET_ERR_CUDA;
   p->in_flight = false;
+  p->n_jobs = 0;  // no statuses to read until this batch is enqueued
   const long long blocks = batch_blocks(p->opts);
   if (blocks < 1) return VOXTET_ERR_CUDA;
   // nothing of this plan is in flight, so the pinned image is free
@@ -1808,20 +1809,20 @@ int voxtet_plan_run(voxtet_plan *p, const voxtet_job *jobs, int32_t n_jobs, void
   const size_t need =
       build_batch_image(jobs, n_jobs, p->cap, p->opts, blocks, p->ws, p->ws_bytes, p->pinned, hs.data());
   if (need > p->ws_bytes) return VOXTET_ERR_NOMEM;
-  p->host_status.swap(hs);
   cudaGraphExec_t &exec = p->exec;
   if (!exec) {  // capture the upload and the kernels once; later runs replay them
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return VOXTET_ERR_CUDA;
-    cudaMemcpyAsync(p->ws, p->pinned, p->image_bytes, cudaMemcpyHostToDevice, p->cap_stream);
+    const cudaError_t up = cudaMemcpyAsync(p->ws, p->pinned, p->image_bytes, cudaMemcpyHostToDevice, p->cap_stream);
     const unsigned long long before = g_launches.load();
     const int st = launch_batch(p->ws, p->cap, p->opts.mode == 1, p->opts.row_cull != 2, p->cap_stream);
     // the jobs' status words come back into the image with the batch
     const size_t o_status = batch_layout(p->cap).o_status;
-    cudaMemcpyAsync(p->pinned + o_status, p->ws + o_status, (size_t)p->cap * sizeof(int), cudaMemcpyDeviceToHost,
-                    p->cap_stream);
+    const cudaError_t down = cudaMemcpyAsync(p->pinned + o_status, p->ws + o_status, (size_t)p->cap * sizeof(int),
+                                             cudaMemcpyDeviceToHost, p->cap_stream);
     g_launches.store(before);  // captured, not launched
-    if (cudaStreamEndCapture(p->cap_stream, &g) != cudaSuccess || st != VOXTET_OK) {
+    if (cudaStreamEndCapture(p->cap_stream, &g) != cudaSuccess || up != cudaSuccess || down != cudaSuccess ||
+        st != VOXTET_OK) {
       if (g) cudaGraphDestroy(g);
       return VOXTET_ERR_CUDA;
     }
@@ -1835,8 +1836,12 @@ int voxtet_plan_run(voxtet_plan *p, const voxtet_job *jobs, int32_t n_jobs, void
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
   if (cudaGraphLaunch(exec, stream) != cudaSuccess) return VOXTET_ERR_CUDA;
   g_launches.fetch_add(kBatchLaunches);
-  if (cudaEventRecord(p->done, stream) != cudaSuccess) return VOXTET_ERR_CUDA;
+  if (cudaEventRecord(p->done, stream) != cudaSuccess) {
+    cudaStreamSynchronize(stream);  // the batch still uses the image and the workspace
+    return VOXTET_ERR_CUDA;
+  }
   p->in_flight = true;
+  p->host_status.swap(hs);
   p->n_jobs = n_jobs;
   return VOXTET_OK;
 }
