@@ -150,8 +150,11 @@ class Plan:
     def run(self, specs: Sequence[JobSpec], stream=None) -> int:
         """Enqueue a batch; returns the status (ERR_NOMEM if it does not fit)."""
         self._jobs = make_jobs(specs)  # keep alive until the table is built
-        self._n = len(specs)
-        return int(self.lib.voxtet_plan_run(self._handle, self._jobs, self._n, vt._stream_ptr(stream)))
+        n = len(specs)
+        st = int(self.lib.voxtet_plan_run(self._handle, self._jobs, n, vt._stream_ptr(stream)))
+        if st != vt.ERR_ARG:  # a refused call leaves the run before it; any other failure leaves none
+            self._n = n if st == vt.OK else 0
+        return st
 
     def done(self) -> bool:
         r = int(self.lib.voxtet_plan_query(self._handle))
@@ -160,6 +163,7 @@ class Plan:
         return r == 1
 
     def wait(self) -> List[int]:
+        """Wait for the last run; its jobs' statuses (none after a run that failed)."""
         arr = (ctypes.c_int32 * max(self._n, 1))()
         st = self.lib.voxtet_plan_wait(self._handle, arr)
         if st != vt.OK:
