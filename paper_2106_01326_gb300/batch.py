@@ -83,16 +83,19 @@ def make_jobs(specs: Sequence[JobSpec]):
     try:
         for sp in specs:
             v, t = sp.mesh.verts, sp.mesh.tets
+            if type(sp.origin) is not tuple:  # numpy's rules: a single number, one for all three, [1, 3]
+                return _make_jobs_converting(specs)
             x, y, z = sp.origin
             rows.append(pack(v.data_ptr(), v.shape[0], t.data_ptr(), t.shape[0], x, y, z, sp.voxel_size, sp.res,
                              sp.span_rows, 0, 0, sp.out.data_ptr()))
-    except (struct.error, OverflowError, TypeError):
+    except (struct.error, OverflowError, TypeError, ValueError):
         return _make_jobs_converting(specs)
     return (vt.Job * max(len(rows), 1)).from_buffer(bytearray(b"".join(rows) or ctypes.sizeof(vt.Job)))
 
 
 def _make_jobs_converting(specs: Sequence[JobSpec]):
-    """The same for values that need numpy's conversions (numbers beyond float32, float sizes)."""
+    """The same for values that need numpy's conversions (numbers beyond float32, float sizes, origins
+    of one number or in other containers than a tuple); refuses what numpy refuses."""
     import numpy as np
 
     rows = [(sp.mesh.verts.data_ptr(), sp.mesh.verts.shape[0], sp.mesh.tets.data_ptr(), sp.mesh.tets.shape[0],

@@ -1,7 +1,9 @@
-"""Host logic of batches, without a GPU: the plan object's bookkeeping (the library is a fake)."""
+"""Host logic of batches, without a GPU: the job table and the plan object's bookkeeping (the library
+is a fake)."""
 import ctypes
 from types import SimpleNamespace
 
+import numpy as np
 import pytest
 import torch
 
@@ -73,3 +75,37 @@ def test_plan_whose_run_raises_keeps_its_last_run(plan):
     with pytest.raises(TypeError):
         plan.run(bad, stream=STREAM)
     assert plan.wait() == [vt.ERR_NAN] * 4
+
+
+def _origin(value):
+    specs = _specs(1)
+    specs[0].origin = value
+    return list(batch.make_jobs(specs)[0].origin)
+
+
+@pytest.mark.parametrize("value,want", [
+    ((1.0, 2.0, 3.0), [1, 2, 3]),
+    ([1, 2, 3], [1, 2, 3]),
+    (np.array([1.0, 2.0, 3.0]), [1, 2, 3]),
+    (torch.tensor([1.0, 2.0, 3.0]), [1, 2, 3]),
+    (1.5, [1.5] * 3),
+    (np.float32(1.5), [1.5] * 3),
+    ((1.5,), [1.5] * 3),
+    (np.array([1.5]), [1.5] * 3),
+    (np.array([[1.0, 2.0, 3.0]]), [1, 2, 3]),
+], ids=str)
+def test_origins_of_a_job(value, want):
+    """A job's origin follows numpy's assignment to three float32 values."""
+    assert _origin(value) == want
+
+
+@pytest.mark.parametrize("value", [(1, 2), (1, 2, 3, 4), {1: 0, 2: 0, 3: 0}], ids=str)
+def test_origins_that_are_refused(value):
+    with pytest.raises((TypeError, ValueError)):
+        _origin(value)
+
+
+def test_one_odd_job_leaves_the_others_alone():
+    specs = _specs(5)
+    specs[3].origin, specs[4].origin = (0.5,), (1.0, 2.0, 3.0)
+    assert [list(j.origin) for j in batch.make_jobs(specs)] == [[0] * 3] * 3 + [[0.5] * 3, [1, 2, 3]]
