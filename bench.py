@@ -301,9 +301,6 @@ def batched_section(args, flush, stream):
         specs.append(batch.JobSpec(m, j.res, vt.alloc_grid(j.res), j.origin, j.voxel_size))
         ref_out.append(vt.alloc_grid(j.res))
     n_tets = sum(len(j.tets) for j in jobs)
-    from paper_2106_01326_gb300 import autotune
-
-    tuned = autotune.tune_batch(specs, reps=2)  # per-resolution span size, untimed
     plan = batch.Plan(batch.batch_workspace_size(specs, len(specs)), len(specs))
     ws_single = [vt.alloc_workspace(sp.mesh.n_tets, sp.mesh.n_verts, sp.res) for sp in specs]
 
@@ -315,7 +312,7 @@ def batched_section(args, flush, stream):
     def run_single(events=None):
         for i, sp in enumerate(specs):
             vt.voxelize(sp.mesh.verts, sp.mesh.tets, sp.origin, sp.voxel_size, sp.res, out=ref_out[i],
-                        workspace=ws_single[i], sync=False, stream=stream, span_rows=sp.span_rows)
+                        workspace=ws_single[i], sync=False, stream=stream)
             if events is not None:
                 events[i].record(stream)
 
@@ -372,7 +369,6 @@ def batched_section(args, flush, stream):
                      "ms_per_batch": smean, "latency_ms_p50": q(s_lat, 50), "latency_ms_p99": q(s_lat, 99),
                      "form": "256 voxelize_tets calls on one stream"},
         "speedup_jobs_per_s": smean / bmean,
-        "span_rows_by_res": {str(r): v["span_rows"] for r, v in tuned.items()},
         "bit_identical": exact,
         "oracle_exact": f"{oracle_ok}/{len(specs)}", "oracle_s": oracle_s, "oracle_threads": oracle.last_threads(),
     }

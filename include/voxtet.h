@@ -246,7 +246,7 @@ typedef struct {
     float origin[3];       /* grid corner (ignored if fixed_point) */
     float voxel_size;      /* > 0 (ignored if fixed_point) */
     int32_t res;           /* power of two in [1, VOXTET_MAX_RES] */
-    int32_t span_rows;     /* bounding-box rows per work item; 0 = opts->span_rows or automatic */
+    int32_t span_rows;     /* checked (0 to 2^20) and otherwise unused: batches run slice units, which have no spans */
     int32_t fixed_point;   /* 1: d_verts holds lattice coordinates as in voxelize_tets_fixed */
     int32_t reserved;
     uint32_t *d_out_bits;  /* DEVICE grid of this job, layout as for voxelize_tets */

@@ -152,8 +152,11 @@ def settings_for(res: int) -> Tuple[int, int, int]:
 
 
 def tune_batch(specs: Iterable, reps: int = 3) -> Dict[int, dict]:
-    """Tune each resolution present in a batch on its largest job, then set every
-    job's span_rows from the result (jobs are ``batch.JobSpec``)."""
+    """Tune each resolution present in a batch on its largest job (jobs are ``batch.JobSpec``).
+
+    Batches run slice units, whose one setting is ``row_cull``, a choice for the whole batch: the
+    results' "row_cull" are candidates for ``batch.Plan`` and ``batch.voxelize_batched``.  Every
+    job's span_rows, which slice units do not use, is set to the results' 0."""
     specs = list(specs)
     by_res: Dict[int, list] = {}
     for sp in specs:
@@ -161,9 +164,8 @@ def tune_batch(specs: Iterable, reps: int = 3) -> Dict[int, dict]:
     out = {}
     for res, group in sorted(by_res.items()):
         big = max(group, key=lambda s: s.mesh.n_tets)
-        # batches run the span kernel (one persistent launch over every job's tiles)
-        out[res] = tune(big.mesh.verts, big.mesh.tets, big.origin, big.voxel_size, res, culls=(0,), reps=reps,
-                        kernels=(vt.KERNEL_SPANS,), store=False)
+        out[res] = tune(big.mesh.verts, big.mesh.tets, big.origin, big.voxel_size, res, reps=reps,
+                        kernels=(vt.KERNEL_SLICES,), store=False)
         for sp in group:
             sp.span_rows = out[res]["span_rows"]
     return out

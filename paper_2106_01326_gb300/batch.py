@@ -44,7 +44,7 @@ class JobSpec:
     out: "object"  # int32 grid tensor [res, res, W]
     origin: Tuple[float, float, float] = (0.0, 0.0, 0.0)
     voxel_size: float = 0.0
-    span_rows: int = 0
+    span_rows: int = 0  # unused by batches (slice units have no spans)
 
     def __post_init__(self):
         if not self.voxel_size:

@@ -131,6 +131,7 @@ class Server:
     ``arena_bytes``: device memory for output grids; a request is admitted only
     when its grid fits.  ``n_slots`` plans (each with ``slot_workspace_bytes`` of
     workspace and its own stream) keep up to that many batches in flight.
+    ``span_rows_by_res`` sets its jobs' span_rows, which batches do not use.
     ``on_result(ticket, grid)`` is called for every finished request before its
     grid's memory is reused (copy the grid out there if it is needed later).
     """

@@ -1,6 +1,7 @@
 """Host logic of the autotuner, without a GPU: candidate choice, the equal-grid check and the
 per-device, per-resolution cache (timings and grids come from a fake)."""
 import json
+import types
 
 import pytest
 import torch
@@ -74,3 +75,19 @@ def test_store_false_leaves_cache_alone(fake, tmp_path):
     r = autotune.tune(v, t, (0, 0, 0), 1 / 128, 128, culls=(1,), store=False, kernels=(1,))
     assert r["span_rows"] == min(autotune.SPAN_CANDIDATES)
     assert not (tmp_path / "tune.json").exists()
+
+
+def test_tune_batch_times_what_a_batch_runs(fake):
+    """A batch runs slice units: only their settings are timed, once per resolution, on the largest
+    job, and no span size is set on the jobs."""
+    fake["times"] = {("slices", 1): 30.0, ("slices", 2): 20.0}
+    v, t = _mesh()
+    jobs = [types.SimpleNamespace(mesh=types.SimpleNamespace(verts=v, tets=t.expand(k, 4), n_tets=k), res=res,
+                                  origin=(0.0, 0.0, 0.0), voxel_size=1 / res, span_rows=256)
+            for k, res in ((1, 64), (7, 64), (2, 32))]
+    r = autotune.tune_batch(jobs)
+    assert sorted(r) == [32, 64]
+    assert [(x["kernel"], x["span_rows"], x["row_cull"], x["n_tets"]) for x in (r[32], r[64])] == [(2, 0, 2, 2),
+                                                                                                 (2, 0, 2, 7)]
+    assert sorted(fake["calls"]) == [("slices", 1), ("slices", 1), ("slices", 2), ("slices", 2)]
+    assert [j.span_rows for j in jobs] == [0, 0, 0]
