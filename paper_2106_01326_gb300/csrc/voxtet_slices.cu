@@ -211,7 +211,7 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, int lg, Su
   if (CULL) {
     row_range(V, bx, p.sh, R);
   } else {
-    R.kL0 = R.kL1 = R.kU0 = R.kU1 = 0.f;
+    R.kL0 = R.kL1 = R.kU0 = R.kU1 = R.z0 = R.z1 = 0.f;
     R.aL0 = R.aL1 = 0.f;
     R.aU0 = R.aU1 = fb;
   }
