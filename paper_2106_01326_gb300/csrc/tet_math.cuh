@@ -146,6 +146,28 @@ __device__ __forceinline__ void exact_setup(const int3 V[4], const Box &bx, int 
   X.Dx[3] = n3x * two_s; X.Dy[3] = n3y * two_s; X.Dz[3] = n3z * two_s;
 }
 
+// Exact affine data of constraint m alone, m = 0..3 a run-time value, of type T as for exact_setup: the
+// faces of slot_exact below.  With coordinates up to 2^21 the normal's components are below 2^45.
+template <typename T>
+__device__ __forceinline__ void face_exact(const int3 V[4], const Box &bx, int sh, int m, T &L, T &Dx, T &Dy, T &Dz) {
+  const int s = 1 << (sh - 1);
+  const int3 A = m == 0 ? V[1] : V[0];
+  const int3 U = m == 2 ? V[3] : m == 3 ? V[1] : V[2];
+  const int3 W = m == 2 ? V[1] : m == 3 ? V[2] : V[3];
+  const i64 ux = U.x - A.x, uy = U.y - A.y, uz = U.z - A.z;
+  const i64 wx = W.x - A.x, wy = W.y - A.y, wz = W.z - A.z;
+  const i64 sg = m == 0 ? -1 : 1;
+  const i64 nx = sg * (uy * wz - uz * wy), ny = sg * (uz * wx - ux * wz), nz = sg * (ux * wy - uy * wx);
+  const i64 qx = (i64)(s + (bx.i0 << sh)) - A.x;
+  const i64 qy = (i64)(s + (bx.j0 << sh)) - A.y;
+  const i64 qz = (i64)(s + (bx.l0 << sh)) - A.z;
+  L = (T)qx * nx + (T)qy * ny + (T)qz * nz;
+  const T two_s = (T)1 << sh;
+  Dx = nx * two_s;
+  Dy = ny * two_s;
+  Dz = nz * two_s;
+}
+
 // Exact affine data of constraint m alone (64-bit, requires E <= 2^20), so that a
 // caller can process one face at a time.  Face m is opposite vertex m:
 //   m = 1, 2, 3:  lam_m(P) = (P - V0) . n_m with n1 = e2 x e3, n2 = e3 x e1, n3 = e1 x e2
@@ -177,44 +199,6 @@ __device__ __forceinline__ void slot_exact(const int3 V[4], const Box &bx, int s
   Dz = nz * two_s;
 }
 
-// Slot of each constraint: first those with Dx < 0 (upper bounds on a), then
-// Dx > 0 (lower bounds), then Dx == 0 (whole-row conditions).  slot[m] is the
-// position of constraint m; nup / nlo count the first two groups.
-template <typename T>
-__device__ __forceinline__ void slot_order(const Exact<T> &X, int slot[4], int &nup, int &nlo) {
-  int up = 0, lo = 0;
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    up += X.Dx[m] < 0;
-    lo += X.Dx[m] > 0;
-  }
-  int cu = 0, cl = up, cz = up + lo;
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    if (X.Dx[m] < 0) slot[m] = cu++;
-    else if (X.Dx[m] > 0) slot[m] = cl++;
-    else slot[m] = cz++;
-  }
-  nup = up;
-  nlo = lo;
-}
-
-// Permute X into slot order (register-friendly: fully unrolled selects).
-template <typename T>
-__device__ __forceinline__ void permute_slots(Exact<T> &X, const int slot[4]) {
-  Exact<T> Y;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    Y.L[q] = 0; Y.Dx[q] = 0; Y.Dy[q] = 0; Y.Dz[q] = 0;
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-      if (slot[m] == q) {
-        Y.L[q] = X.L[m]; Y.Dx[q] = X.Dx[m]; Y.Dy[q] = X.Dy[m]; Y.Dz[q] = X.Dz[m];
-      }
-  }
-  X = Y;
-}
-
 template <bool STRICT, typename T>
 __device__ __forceinline__ bool lam_ok(T v) {
   return STRICT ? (v > 0) : (v >= 0);
@@ -222,7 +206,8 @@ __device__ __forceinline__ bool lam_ok(T v) {
 
 // Exact sample interval [lo, hi] (0-based within the box's x-extent na) of row (b, c);
 // returns false if the row has no sample.  Each bound is found by bisection on the
-// monotone exact lam(a) = H + Dx a, probing only a in [0, na-1] (inside the box).
+// monotone exact lam(a) = H + Dx a, probing only a in [0, na-1] (inside the box).  X's faces in slot order:
+// nup with Dx < 0 (upper bounds on a), nlo with Dx > 0 (lower bounds), then those with Dx = 0.
 template <bool STRICT, typename T>
 __device__ __forceinline__ bool exact_row(const Exact<T> &X, int nup, int nlo, int na, int b, int c, int &lo_out,
                                        int &hi_out) {

@@ -715,16 +715,41 @@ __global__ void __launch_bounds__(kListBlock) k_slab_list(Params p) {
 // ------------------------------------------------------------------ the exact kernel
 
 constexpr int kExactBlock = 128;
+constexpr int kExactBlocksPerSM = 7;  // 72 registers a thread
 
-// Every bounding-box row of tet t, solved with exact integers of type T by the
-// threads of one block (threads stride over the rows).
+// A tet's exact face data in shared memory (Exact<i64> or Exact<i128>), faces in slot order.
+struct ExactTet {
+  __align__(16) unsigned char x[sizeof(Exact<i128>)];
+  int nup, nlo;
+};
+
+// Every bounding-box row of a tet, solved with exact integers of type T by the threads of one block
+// (threads stride over the rows).  Four threads set up a face each, and all read the faces from shared
+// memory: held by every thread they took 147 registers, which left three blocks per SM to this work and
+// to the queued rows in the same kernel.
 template <bool STRICT, typename T>
-__device__ __forceinline__ void exact_tet_rows(const Params &p, const int3 V[4], const Box &bx) {
-  Exact<T> X;
-  exact_setup<T>(V, bx, p.sh, X);
-  int slot[4], nup = 0, nlo = 0;
-  slot_order<T>(X, slot, nup, nlo);
-  permute_slots<T>(X, slot);
+__device__ __forceinline__ void exact_tet_rows(const Params &p, const int3 V[4], const Box &bx, ExactTet &sm) {
+  Exact<T> &X = *reinterpret_cast<Exact<T> *>(sm.x);
+  __syncthreads();  // the previous tet's rows are solved
+  if (threadIdx.x < 32) {
+    const int m = threadIdx.x & 3;
+    T L, Dx, Dy, Dz;
+    face_exact<T>(V, bx, p.sh, m, L, Dx, Dy, Dz);
+    // slots: faces with Dx < 0 (upper bounds on a), then Dx > 0 (lower bounds), then Dx = 0
+    const unsigned up = __ballot_sync(0xFFFFFFFFu, Dx < 0) & 15u, lo = __ballot_sync(0xFFFFFFFFu, Dx > 0) & 15u;
+    const unsigned below = (1u << m) - 1u, mine = Dx < 0 ? up : Dx > 0 ? lo : ~(up | lo);
+    const int q = __popc(mine & below) + (Dx < 0 ? 0 : __popc(up)) + (Dx == 0 ? __popc(lo) : 0);
+    if (threadIdx.x < 4) {
+      X.L[q] = L;
+      X.Dx[q] = Dx;
+      X.Dy[q] = Dy;
+      X.Dz[q] = Dz;
+      sm.nup = __popc(up);
+      sm.nlo = __popc(lo);
+    }
+  }
+  __syncthreads();
+  const int nup = sm.nup, nlo = sm.nlo;
   const unsigned long long rows = (unsigned long long)bx.nb * (unsigned long long)bx.nc;
   for (unsigned long long r = threadIdx.x; r < rows; r += blockDim.x) {
     const int c = (int)(r / (unsigned long long)bx.nb), b = (int)(r - (unsigned long long)c * bx.nb);
@@ -736,13 +761,14 @@ __device__ __forceinline__ void exact_tet_rows(const Params &p, const int3 V[4],
   }
 }
 
+// Tet t by the threads of one block, all of which call this.
 template <bool STRICT>
-__device__ __forceinline__ void exact_tet(const Params &p, long long t) {
+__device__ __forceinline__ void exact_tet(const Params &p, long long t, ExactTet &sm) {
   int3 V[4];
   Box bx;
   const int E = oriented_tet(p, t, V, bx);
-  if (E <= kNarrowExtent) exact_tet_rows<STRICT, i64>(p, V, bx);
-  else exact_tet_rows<STRICT, i128>(p, V, bx);
+  if (E <= kNarrowExtent) exact_tet_rows<STRICT, i64>(p, V, bx, sm);
+  else exact_tet_rows<STRICT, i128>(p, V, bx, sm);
 }
 
 template <bool STRICT>
@@ -761,17 +787,16 @@ __device__ __forceinline__ void exact_queued_row(const Params &p, const RowItem 
 
 // The tets flagged in the redo bitmap (after a row-queue overflow), by blocks bi of bn.
 template <bool STRICT>
-__device__ __forceinline__ void exact_redo(const Params &p, unsigned bi, unsigned bn) {
+__device__ __forceinline__ void exact_redo(const Params &p, unsigned bi, unsigned bn, ExactTet &sm) {
   for (long long t = bi; t < p.n_tets; t += bn)
-    if ((p.redo[t >> 5] >> (t & 31)) & 1u) exact_tet<STRICT>(p, t);
+    if ((p.redo[t >> 5] >> (t & 31)) & 1u) exact_tet<STRICT>(p, t, sm);
 }
 
 // The queued rows (a thread each), the queued tets (a block each) and, after a row-queue overflow,
-// the flagged ones.  One kernel for all: the 128-bit tet path's registers leave three blocks per SM,
-// 58,368 threads, more than there are queued rows at most sizes (2.3k at 512^3, 20k at 1024^3 for the
-// sliver mesh), and a launch of its own for the rows cost a call 3-4 us.
+// the flagged ones, in one kernel: a launch of its own for the rows cost a call 3-4 us.
 template <bool STRICT>
-__global__ void __launch_bounds__(128) k_exact(Params p) {
+__global__ void __launch_bounds__(kExactBlock, kExactBlocksPerSM) k_exact(Params p) {
+  __shared__ ExactTet sm;
   // no early release of the next kernel: the brick count's blocks, placed unevenly while these run,
   // took 15 us longer per slab
   chain_wait();  // every row and tet is queued
@@ -784,10 +809,11 @@ __global__ void __launch_bounds__(128) k_exact(Params p) {
     if ((threadIdx.x & 31) == 0 && err) atomicOr(&p.hdr->status_bits, err);
   }
   const unsigned n_rq = min(p.hdr->rowq_count, p.q_cap), threads = gridDim.x * blockDim.x;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n_rq; i += threads) exact_queued_row<STRICT>(p, p.rowq[i]);
+  // 64-bit indices: a queue may hold up to 2^32 - 1 entries
+  for (u64 i = blockIdx.x * blockDim.x + threadIdx.x; i < n_rq; i += threads) exact_queued_row<STRICT>(p, p.rowq[i]);
   const unsigned n_tq = min((unsigned long long)p.hdr->tetq_count, (unsigned long long)p.n_tets);
-  for (unsigned q = blockIdx.x; q < n_tq; q += gridDim.x) exact_tet<STRICT>(p, p.tetq[q]);
-  if (p.hdr->rowq_count > p.q_cap) exact_redo<STRICT>(p, blockIdx.x, gridDim.x);
+  for (u64 q = blockIdx.x; q < n_tq; q += gridDim.x) exact_tet<STRICT>(p, p.tetq[q], sm);
+  if (p.hdr->rowq_count > p.q_cap) exact_redo<STRICT>(p, blockIdx.x, gridDim.x, sm);
 }
 
 // ------------------------------------------------------------------ batched kernels
@@ -922,7 +948,9 @@ __device__ __forceinline__ int queue_job(const u64 *pre, int m, u64 x) {
 // spread over all blocks: which jobs' rows need exact work is known only now (a job of wide tets on
 // a fine grid queues many times the rows of one with as many small tets).
 template <bool STRICT>
-__global__ void __launch_bounds__(128) k_exact_batched(const BatchHeader *bh, const JobDesc *jobs) {
+__global__ void __launch_bounds__(kExactBlock, kExactBlocksPerSM) k_exact_batched(const BatchHeader *bh,
+                                                                                  const JobDesc *jobs) {
+  __shared__ ExactTet sm;
   __shared__ u64 pre[kQueueJobs + 1];
   chain_wait();  // every row and tet is queued
   const int n = bh->n_jobs;
@@ -949,14 +977,14 @@ __global__ void __launch_bounds__(128) k_exact_batched(const BatchHeader *bh, co
     for (u64 i = blockIdx.x; i < pre[m]; i += gridDim.x) {
       const int j = queue_job(pre, m, i);
       const Params &p = jobs[j0 + j].p;
-      exact_tet<STRICT>(p, p.tetq[i - pre[j]]);
+      exact_tet<STRICT>(p, p.tetq[i - pre[j]], sm);
     }
     queue_prefix(pre, m, [&](int j) {
       const Params &p = jobs[j0 + j].p;
       return p.hdr->rowq_count > p.q_cap ? 1u : 0u;
     });
     for (int j = 0; pre[m] && j < m; ++j)
-      if (pre[j + 1] > pre[j]) exact_redo<STRICT>(jobs[j0 + j].p, blockIdx.x, gridDim.x);
+      if (pre[j + 1] > pre[j]) exact_redo<STRICT>(jobs[j0 + j].p, blockIdx.x, gridDim.x, sm);
   }
 }
 
