@@ -239,14 +239,21 @@ __device__ __forceinline__ void slice_rows_sorted(const EdgeLines &E, int Z, int
 }
 
 // Queue row (b, c) of tet t for the exact kernel; if the row queue is full, flag the
-// whole tet for an exact redo instead.
+// whole tet for an exact redo instead.  TOGETHER: one atomic for the lanes that are here at once,
+// for blocks with a small stage; the span kernel, whose stage seldom overflows, has no registers for
+// it (80 more bytes spilled, sliver mesh at 512^3 349 -> 361 us a call).
+template <bool TOGETHER>
 __device__ __forceinline__ void queue_row(const Params &p, long long t, int b, int c) {
-  // one atomic for the lanes that are here together
-  const unsigned m = __activemask(), lane = threadIdx.x & 31;
-  const int first = __ffs(m) - 1;
-  unsigned k = 0;
-  if ((int)lane == first) k = atomicAdd(&p.hdr->rowq_count, (unsigned)__popc(m));
-  k = __shfl_sync(m, k, first) + (unsigned)__popc(m & ((1u << lane) - 1u));
+  unsigned k;
+  if (TOGETHER) {
+    const unsigned m = __activemask(), lane = threadIdx.x & 31;
+    const int first = __ffs(m) - 1;
+    k = 0;
+    if ((int)lane == first) k = atomicAdd(&p.hdr->rowq_count, (unsigned)__popc(m));
+    k = __shfl_sync(m, k, first) + (unsigned)__popc(m & ((1u << lane) - 1u));
+  } else {
+    k = atomicAdd(&p.hdr->rowq_count, 1u);
+  }
   if (k < p.q_cap) {
     RowItem it;
     it.tet = (uint32_t)t;
@@ -309,7 +316,7 @@ __device__ __forceinline__ void queue_row_staged(const Params &p, RowStageN<N> &
     it.c = (uint16_t)c;
     st.items[k] = it;
   } else {
-    queue_row(p, t, b, c);
+    queue_row<(N < kStage)>(p, t, b, c);
   }
 }
 

@@ -59,3 +59,26 @@ def test_mixed_widths(vt, n, wide, res, mode):
         assert st["wide_tets"] == 0 or wide > 0
         if not use_filter:
             assert st["exact_tets"] > 0.4 * n
+
+
+@pytest.mark.parametrize("kernel", [1, 2], ids=["spans", "slices"])
+@pytest.mark.parametrize("n,res", [(4, 32), (6, 128), (12, 128)])
+def test_rows_queued_past_a_blocks_stage(vt, n, res, kernel):
+    """Cells of 4:12:12, whose faces meet sample centres every third row: each tile queues many times the
+    rows a block stages (512 in the span kernel, 64 in the slice-unit kernel), the largest mesh more
+    than the row queue holds, so that whole tets are solved again."""
+    import torch
+
+    from paper_2106_01326_gb300 import meshgen as mg
+
+    ijk, tets = mg.kuhn_lattice_int(n)
+    half = L // 2 // res
+    unit = max(1, L // (12 * n) // (2 * half // 8)) * (2 * half // 8)
+    xyz = (ijk * (np.array([4, 12, 12]) * unit) + half).astype(np.int32)
+    ref = oracle.voxelize_fixed(xyz, tets, res)
+    x, t = torch.from_numpy(xyz).cuda(), torch.from_numpy(tets).cuda()
+    ws = vt.alloc_workspace(len(tets), len(xyz), res)
+    got = vt.voxelize_fixed(x, t, res, workspace=ws, kernel=kernel)
+    assert np.array_equal(got.cpu().numpy().view(np.uint32).reshape(ref.shape), ref)
+    queued = vt.read_stats(ws)["fallback_rows"]
+    assert queued > 512 and (n < 12 or queued > 65536)
