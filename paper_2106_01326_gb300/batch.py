@@ -82,10 +82,11 @@ def make_jobs(specs: Sequence[JobSpec]):
     rows = []
     try:
         for sp in specs:
-            v, t = sp.mesh.verts, sp.mesh.tets
-            if type(sp.origin) is not tuple:  # numpy's rules: a single number, one for all three, [1, 3]
+            mesh, origin = sp.mesh, sp.origin
+            v, t = mesh.verts, mesh.tets
+            if type(origin) is not tuple:  # numpy's rules: a single number, one for all three, [1, 3]
                 return _make_jobs_converting(specs)
-            x, y, z = sp.origin
+            x, y, z = origin
             rows.append(pack(v.data_ptr(), v.shape[0], t.data_ptr(), t.shape[0], x, y, z, sp.voxel_size, sp.res,
                              sp.span_rows, 0, 0, sp.out.data_ptr()))
     except (struct.error, OverflowError, TypeError, ValueError):

@@ -352,9 +352,8 @@ struct TileCounters {
 };
 
 
-// Adds a block's counters to a mesh's header: one atomic per warp and counter.  Error bits also
-// go to `status` if one is given (a batch job's status word).
-__device__ __forceinline__ void flush_counters(Header *hdr, TileCounters &ctr, int *status = nullptr) {
+// Adds a block's counters to a mesh's header: one atomic per warp and counter.
+__device__ __forceinline__ void flush_counters(Header *hdr, TileCounters &ctr) {
   const int lane = threadIdx.x & 31;
   unsigned long long rows_w = ctr.rows, deg_w = ctr.degenerate, wide_w = ctr.wide;
 #pragma unroll
@@ -369,7 +368,6 @@ __device__ __forceinline__ void flush_counters(Header *hdr, TileCounters &ctr, i
     if (deg_w) atomicAdd(&hdr->degenerate, deg_w);
     if (wide_w) atomicAdd(&hdr->wide, wide_w);
     if (err) atomicOr(&hdr->status_bits, err);
-    if (err && status) atomicOr(status, err);
   }
   if (threadIdx.x == 0 && ctr.spans) atomicAdd(&hdr->spans, ctr.spans);
   ctr = TileCounters();

@@ -17,7 +17,7 @@
 //       voxtet_rows.cuh), and the interval ORed into the grid's words.
 // Where a mesh has too few tets for a thread each to fill the chip, or tets of more slices than a
 // thread takes, a group of 2^lg threads shares a tet and its slices (su_group_log2); slices or rows
-// past that are taken in further windows of the same tile.  A batch's jobs run in one launch
+// past that are taken in further windows of the same tile, by the tets that have them.  A batch's jobs run in one launch
 // (k_slices_batched), a thin slab's tets from a list (LIST).
 // What bounds it: instruction issue and, on finer grids, the rate at which ORs reach L2, half of
 // them across the dies.  Measured on GB300 with timing-only copies, 1.3 M-tet sliver mesh: at
@@ -71,6 +71,15 @@ struct SuSmem {
   long long tile;
   int c0, r0;            // the current window: slices from c0, rows from r0 of each tet's box
   int next_c0, next_r0;  // the window after it (0, 0: the tile is done)
+  // the current window's tets, 2^lg threads each: all of the tile (n_sel = 0, lg = tile_lg) or the
+  // n_sel at places place[buf] of it; those of the next window are collected in the other list.
+  // (Read from here where they are used: held across the phases they cost the row loop registers.)
+  int lg, tile_lg, n_sel, n_next, buf;
+  uint8_t place[2][kSuBlock];
+  // the block's counters but for the rows, since the last flush
+  unsigned long long spans;
+  unsigned degenerate, wide;
+  int err;
 };
 
 // 16-slice tiles fit 7 blocks per SM (228 KB, 1 KB reserved per block), 32-slice tiles 5
@@ -88,29 +97,33 @@ __device__ __forceinline__ int su_counter(int n, int w) {
 // to sm.slice (0 if none); counts each unit in its counter (no rank is needed here, so the
 // count does not wait on the shared-memory atomic).  `more` is set if the tet has slices past
 // the window; a window also covers at most kSuRows rows per slice, from row r0 of the box, and
-// `tall` is set if the tet's box has rows past it.  A tet is counted (or queued) once, by its
-// group's first thread in its first window.
+// `tall` is set if the tet's box has rows past it (both alike for all threads of a group).  A tet is
+// counted (or queued) once, by its group's first thread in its first window; zero-volume and wide
+// tets and errors, all rare, in shared memory, so that the counters take no registers.
 template <bool STRICT, bool CULL, bool TALL, int SL>
-__device__ __forceinline__ int su_setup(const Params &p, long long t, int lg, SuSmem<SL> &sm, TileCounters &ctr,
-                                        bool &more, bool &tall) {
+__device__ __forceinline__ int su_setup(const Params &p, long long t, SuSmem<SL> &sm, bool &more, bool &tall) {
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int sub = tid & ((1 << lg) - 1);
-  const int c0 = sm.c0, r0 = TALL ? sm.r0 : 0;
-  const bool first = (sub | c0 | r0) == 0;
   if (t < 0) return 0;
+  const int lg = sm.lg;
+  const bool first = ((tid & ((1 << lg) - 1)) | sm.c0 | (TALL ? sm.r0 : 0)) == 0;
   int3 V[4];
-  if (!load_tet(p, t, V, ctr.err)) return 0;
+  {
+    int err = 0;
+    const bool valid = load_tet(p, t, V, err);
+    if (err) atomicOr(&sm.err, err);
+    if (!valid) return 0;
+  }
   Box bx;
   const int E = tet_box(V, p.sh, p.rx, p.ry, p.z0, p.z1, bx);
   const bool empty = bx.na <= 0 || bx.nb <= 0 || bx.nc <= 0;
   if (E > kNarrowExtent) {  // wider than 2^20 lattice units: 128-bit sign, exact kernel
     if (!first) return 0;
     if (v6_sign(V, E) == 0) {
-      ++ctr.degenerate;
+      atomicAdd(&sm.degenerate, 1u);
       return 0;
     }
     if (empty) return 0;
-    ++ctr.wide;
+    atomicAdd(&sm.wide, 1u);
     const unsigned k = atomicAdd(&p.hdr->tetq_count, 1u);
     p.tetq[k] = (uint32_t)t;
     return 0;
@@ -124,7 +137,7 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, int lg, Su
   i64 n3x = (i64)e1y * e2z - (i64)e1z * e2y, n3y = (i64)e1z * e2x - (i64)e1x * e2z, n3z = (i64)e1x * e2y - (i64)e1y * e2x;
   i64 v6 = (i64)e1x * n1x + (i64)e1y * n1y + (i64)e1z * n1z;
   if (v6 == 0) {
-    ctr.degenerate += first;
+    if (first) atomicAdd(&sm.degenerate, 1u);
     return 0;
   }
   if (empty) return 0;
@@ -134,7 +147,7 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, int lg, Su
     p.tetq[k] = (uint32_t)t;
     return 0;
   }
-  tall = TALL && bx.nb > r0 + kSuRows;
+  tall = TALL && bx.nb > sm.r0 + kSuRows;
   // Orientation (Lemma 1.1): for V6 < 0 every orientation value of an inside point is <= 0,
   // so negating the normals (and V6) gives the positively oriented form of the same faces.
   if (v6 < 0) {
@@ -215,6 +228,8 @@ __device__ __forceinline__ int su_setup(const Params &p, long long t, int lg, Su
     R.aL0 = R.aL1 = 0.f;
     R.aU0 = R.aU1 = fb;
   }
+  const int c0 = sm.c0, r0 = TALL ? sm.r0 : 0;
+  const int sub = tid & ((1 << lg) - 1);
   const float row0 = (float)r0, row1 = TALL ? fminf(fb, (float)(r0 + kSuRows - 1)) : fb;
   const uint32_t row0_bits = kMagicBits + (uint32_t)r0;
   const int step = 1 << lg, k_end = min(bx.nc, c0 + (SL << lg));
@@ -275,9 +290,22 @@ __device__ __forceinline__ long long su_tet(const Params &p, long long i, long l
   return LIST ? (long long)p.tetq[p.n_tets - 1 - i] : i;
 }
 
-// Phase (3): rows b0 .. b0 + n - 1 of slice k of the tet in `slot` (place t of the launch).
+// Place in the tile of the tet whose threads in the current window include `slot`.
+template <int SL>
+__device__ __forceinline__ int su_place(const SuSmem<SL> &sm, int slot) {
+  const int g = slot >> sm.lg;
+  return sm.n_sel ? (int)sm.place[sm.buf][g] : g;
+}
+
+// ... and in the launch.
+template <int SL>
+__device__ __forceinline__ long long su_launch_place(const SuSmem<SL> &sm, int slot) {
+  return sm.tile * (kSuBlock >> sm.tile_lg) + su_place(sm, slot);
+}
+
+// Phase (3): rows b0 .. b0 + n - 1 of slice k of the tet in `slot`.
 template <bool STRICT, bool PAIRS, bool LIST, bool BATCH, int SL>
-__device__ __forceinline__ void su_walk(const Params &p, SuSmem<SL> &sm, int slot, long long t, int k, int b0, int n) {
+__device__ __forceinline__ void su_walk(const Params &p, SuSmem<SL> &sm, int slot, int k, int b0, int n) {
   const float4 *R = reinterpret_cast<const float4 *>(sm.rec + slot * kSuRec);
   const float4 qa = R[0], qb = R[1], qg = R[2], qi = R[3];
   const float cf = (float)k, INF = __int_as_float(0x7f800000);
@@ -329,32 +357,43 @@ __device__ __forceinline__ void su_walk(const Params &p, SuSmem<SL> &sm, int slo
     while (amb) {
       const int j = __ffs(amb) - 1;
       amb &= amb - 1u;
-      queue_row_staged(p, sm.stage, su_tet<LIST>(p, t, p.n_tets), b0 + s1 - 1 - j, k);
+      queue_row_staged(p, sm.stage, su_tet<LIST>(p, su_launch_place(sm, slot), p.n_tets), b0 + s1 - 1 - j, k);
     }
   }
 }
 
-// Phases (1)-(3) of one window of a tile: the tets at places base .. base + (kSuBlock >> lg) - 1
-// (those below `end`), each shared by a group of 2^lg threads.  All threads of the block call it,
-// in step.  The caller's
-// loop claims a tile or moves to the tile's next window: a loop of its own around these phases
-// cost the row loop its reconvergence (measured on GB300, sliver mesh at 512^3: 26.7 -> 15.9
-// active lanes, 262 -> 440 us).
+// Phases (1)-(3) of one window of tile sm.tile.  The first window holds its kSuBlock >> tile_lg tets
+// (those at places below `end`), 2^tile_lg threads each; a further one the tets with slices or rows
+// past the window before, by as many threads each as there are for them.  (A few wide tets among many
+// small ones would else leave most of the block idle in window after window, with all tets set up
+// again in each: 20 tets of 300-500 slices next to each other in a 663,000-tet mesh at 512^3 1726 ->
+// 1145 us, 20 such tets spread over it 725 -> 332.)
+// All threads of the block call it, in step; if it returns true, su_next_window is to be asked before
+// another tile is claimed.  The caller's loop claims a tile or moves to the tile's next window: a loop
+// of its own around these phases cost the row loop its reconvergence (measured on GB300, sliver mesh
+// at 512^3: 26.7 -> 15.9 active lanes, 262 -> 440 us).
 template <bool STRICT, bool CULL, bool PAIRS, bool TALL, bool LIST, bool BATCH, int SL>
-__device__ __forceinline__ void su_pass(const Params &p, long long base, long long end, int lg, SuSmem<SL> &sm,
-                                        TileCounters &ctr) {
+__device__ __forceinline__ bool su_pass(const Params &p, long long end, SuSmem<SL> &sm, unsigned &rows) {
   const int tid = threadIdx.x;
   // (1) set up this thread's tet and its slices' row ranges; count units per counter
   bool more = false, tall = false;
-  const long long t = su_tet<LIST>(p, base + (tid >> lg), end);
-  const int nc = su_setup<STRICT, CULL, TALL, SL>(p, t, lg, sm, ctr, more, tall);
+  const int n_sel = sm.n_sel, lg = sm.lg;
+  int g = tid >> lg;
+  const bool any = n_sel == 0 || g < n_sel;
+  if (n_sel && any) g = sm.place[sm.buf][g];
+  const long long t = any ? su_tet<LIST>(p, sm.tile * (kSuBlock >> (n_sel ? sm.tile_lg : lg)) + g, end) : -1;
+  const int nc = su_setup<STRICT, CULL, TALL, SL>(p, t, sm, more, tall);
+  bool again;
   {
     const bool any_more = __syncthreads_or(more);
     const bool any_tall = TALL && p.ry > kSuRows && __syncthreads_or(tall);
+    again = any_more || any_tall || n_sel;
+    if ((more || tall) && (tid & ((1 << sm.lg) - 1)) == 0)
+      sm.place[sm.buf ^ 1][atomicAdd(&sm.n_next, 1)] = (uint8_t)su_place(sm, tid);
     if (tid == 0) {
       sm.stage.n = 0;  // flushed by the previous window; every thread has passed a barrier since
       // every slice of these rows first, then the next rows
-      sm.next_c0 = any_more ? sm.c0 + (SL << lg) : 0;
+      sm.next_c0 = any_more ? sm.c0 + (SL << sm.lg) : 0;
       if (TALL) sm.next_r0 = any_more ? sm.r0 : any_tall ? sm.r0 + kSuRows : 0;
     }
   }
@@ -375,7 +414,7 @@ __device__ __forceinline__ void su_pass(const Params &p, long long base, long lo
     sm.unit[pos] = (uint32_t)tid | ((uint32_t)k << 7) | (e << 12);
   }
   __syncthreads();
-  if (tid == 0) ctr.spans += total;
+  if (tid == 0) sm.spans += total;
   sm.hist[2 * tid] = 0u;  // ready for the next tile's counts (a barrier comes before them)
   sm.hist[2 * tid + 1] = 0u;
   // (3) walk the units, longest first; a warp takes 32 neighbouring units of the order
@@ -385,27 +424,61 @@ __device__ __forceinline__ void su_pass(const Params &p, long long base, long lo
     const int slot = (int)(u & 127u);
     const int k = c0 + ((int)((u >> 7) & 31u) << lg) + (slot & ((1 << lg) - 1));
     const int b0 = (int)((u >> 12) & 1023u) + r0, n = (int)(u >> 22) + 1;
-    ctr.rows += (unsigned)n;
-    su_walk<STRICT, PAIRS, LIST, BATCH, SL>(p, sm, slot, base + (slot >> lg), k, b0, n);
+    rows += (unsigned)n;
+    su_walk<STRICT, PAIRS, LIST, BATCH, SL>(p, sm, slot, k, b0, n);
   }
   flush_stage(p, sm.stage);
+  return again;
 }
 
-// The block's first thread moves to the tile's next window; true if the tile is done and
-// another is to be claimed.
+// The block's first thread moves to the tile's next window, after su_pass returned true; true if the
+// tile is done.
 template <int SL>
 __device__ __forceinline__ bool su_next_window(SuSmem<SL> &sm) {
+  const int n = sm.n_next;  // 0: the tile is done
   sm.c0 = sm.next_c0;
   sm.r0 = sm.next_r0;
-  return (sm.c0 | sm.r0) == 0;
+  sm.n_sel = n;
+  sm.n_next = 0;
+  sm.buf ^= 1;
+  sm.lg = n ? __clz(n - 1) - (32 - kSuMaxGroup) : sm.tile_lg;  // the most with n << lg <= kSuBlock
+  return n == 0;
 }
 
 template <int SL>
-__device__ __forceinline__ void su_begin(SuSmem<SL> &sm) {
+__device__ __forceinline__ void su_begin(SuSmem<SL> &sm, int tile_lg) {
   for (int i = threadIdx.x; i < kSuCounters; i += kSuBlock) sm.hist[i] = 0u;
   if (threadIdx.x == 0) {
     sm.stage.n = 0;
-    sm.next_c0 = sm.next_r0 = 0;
+    sm.c0 = sm.r0 = sm.next_c0 = sm.next_r0 = 0;
+    sm.n_sel = sm.n_next = sm.buf = 0;
+    sm.lg = sm.tile_lg = tile_lg;
+    sm.spans = 0;
+    sm.degenerate = sm.wide = 0u;
+    sm.err = 0;
+  }
+}
+
+// Adds the block's counters to a mesh's header (and its error bits to `status`) and resets them.  All
+// threads call it, a barrier after the counted work and one before the next.
+template <int SL>
+__device__ __forceinline__ void su_flush(Header *hdr, SuSmem<SL> &sm, unsigned &rows, int *status = nullptr) {
+  unsigned long long sum = rows;
+  rows = 0;
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) sum += __shfl_down_sync(0xFFFFFFFFu, sum, d);
+  if ((threadIdx.x & 31) == 0 && sum) atomicAdd(&hdr->rows, sum);
+  if (threadIdx.x == 0) {
+    if (sm.spans) atomicAdd(&hdr->spans, sm.spans);
+    if (sm.degenerate) atomicAdd(&hdr->degenerate, (unsigned long long)sm.degenerate);
+    if (sm.wide) atomicAdd(&hdr->wide, (unsigned long long)sm.wide);
+    if (sm.err) {
+      atomicOr(&hdr->status_bits, sm.err);
+      if (status) atomicOr(status, sm.err);
+    }
+    sm.spans = 0;
+    sm.degenerate = sm.wide = 0u;
+    sm.err = 0;
   }
 }
 
@@ -427,26 +500,25 @@ __global__ void __launch_bounds__(kSuBlock, SL == kSuSlicesSmall ? 7 : 5) k_slic
   chain_release();
   extern __shared__ __align__(16) unsigned char su_dyn_smem[];
   SuSmem<SL> &sm = *reinterpret_cast<SuSmem<SL> *>(su_dyn_smem);
-  TileCounters ctr;
-  su_begin(sm);
+  unsigned rows = 0;
   const long long end = LIST ? (long long)p.hdr->listq_count : p.n_tets;
   int lg = p.lg;
   if (LIST && end > 0) {  // as su_group_log2, with the slab's tets counted and their rows added up
-    const float slab = (float)(p.z1 - p.z0), rows = 0.5f * (float)p.hdr->list_rows / (float)end;
+    const float slab = (float)(p.z1 - p.z0), per_tet = 0.5f * (float)p.hdr->list_rows / (float)end;
     while (lg < kSuMaxGroup && (float)(1 << lg) < slab &&
            (((end << lg) / kSuBlock) * 2 < (long long)gridDim.x ||
-            su_share_more((end << lg) / kSuBlock, (long long)gridDim.x, rows, lg)))
+            su_share_more((end << lg) / kSuBlock, (long long)gridDim.x, per_tet, lg)))
       ++lg;
   }
-  
+  su_begin(sm, lg);
+  bool again = false;
   for (;;) {
-    if (threadIdx.x == 0 && su_next_window(sm)) sm.tile = (long long)atomicAdd(&p.hdr->tile_counter, 1ull);
+    if (threadIdx.x == 0 && (!again || su_next_window(sm))) sm.tile = (long long)atomicAdd(&p.hdr->tile_counter, 1ull);
     __syncthreads();
-    const long long base = sm.tile * (kSuBlock >> lg);
-    if (base >= end) break;
-    su_pass<STRICT, CULL, PAIRS, SL == kSuSlices, LIST, false, SL>(p, base, end, lg, sm, ctr);
+    if (sm.tile * (kSuBlock >> sm.tile_lg) >= end) break;
+    again = su_pass<STRICT, CULL, PAIRS, SL == kSuSlices, LIST, false, SL>(p, end, sm, rows);
   }
-  flush_counters(p.hdr, ctr);
+  su_flush(p.hdr, sm, rows);
 }
 
 // The tiles of every job of a batch, claimed from one counter bh->chunk at a time; a claim's job is
@@ -465,11 +537,12 @@ __global__ void __launch_bounds__(kSuBlock, 7) k_slices_batched(BatchHeader *bh,
   // the current tile, the claim's end, and the current job's first tile and the one after its last
   __shared__ unsigned long long at, claim_end, job_first, job_end;
   const int tid = threadIdx.x;
-  TileCounters ctr;
-  su_begin(sm);
+  unsigned rows = 0;
+  su_begin(sm, 0);
   const int n = bh->n_jobs;
   const unsigned long long total = bh->total_tiles, chunk = bh->chunk;
   int cur = -1;
+  bool again = false;
   if (tid == 0) {
     at = claim_end = job_first = job_end = 0;
     job_s = -1;
@@ -478,7 +551,7 @@ __global__ void __launch_bounds__(kSuBlock, 7) k_slices_batched(BatchHeader *bh,
     if (tid < 32) {
       unsigned long long tile = 0;
       int search = 0;
-      if (tid == 0 && su_next_window(sm)) {
+      if (tid == 0 && (!again || su_next_window(sm))) {
         if (++at >= claim_end) {
           at = atomicAdd(&bh->tile_counter, chunk);
           claim_end = at + chunk;
@@ -504,16 +577,17 @@ __global__ void __launch_bounds__(kSuBlock, 7) k_slices_batched(BatchHeader *bh,
     const int j = job_s;
     if (j < 0) break;
     if (j != cur) {  // a new job: flush the previous job's counters, load its Params
-      if (cur >= 0) flush_counters(sp.hdr, ctr, status + cur);
+      if (cur >= 0) su_flush(sp.hdr, sm, rows, status + cur);
       __syncthreads();
       if (tid < (int)(sizeof(Params) / sizeof(uint32_t)))
         reinterpret_cast<uint32_t *>(&sp)[tid] = reinterpret_cast<const uint32_t *>(&jobs[j].p)[tid];
+      if (tid == 0) sm.lg = sm.tile_lg = jobs[j].p.lg;  // a new job's tile is at its first window
       __syncthreads();
       cur = j;
     }
-    su_pass<STRICT, CULL, false, true, false, true, SL>(sp, sm.tile * (kSuBlock >> sp.lg), sp.n_tets, sp.lg, sm, ctr);
+    again = su_pass<STRICT, CULL, false, true, false, true, SL>(sp, sp.n_tets, sm, rows);
   }
-  if (cur >= 0) flush_counters(sp.hdr, ctr, status + cur);
+  if (cur >= 0) su_flush(sp.hdr, sm, rows, status + cur);
 }
 
 // ------------------------------------------------------------------ host side

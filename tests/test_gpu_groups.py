@@ -164,3 +164,54 @@ def test_rows_in_pairs_of_words(vt, rx, shift, mode):
     out = store[shift:shift + dims[1] * dims[2] * w].view(dims[2], dims[1], w)
     _same(vt.voxelize_grid(v, t, (0, 0, 0), h, dims, out=out, mode=mode), ref, (rx, shift))
     assert bool((store[:shift] == -1).all()) and bool((store[shift + ref.size:] == -1).all())
+
+
+def _wide_among_small(seed, n, res, wide, lo, hi, where, axis_scale=(1.0, 1.0, 1.0)):
+    """n tets of a few voxels with `wide` of lo..hi voxels: at the end, the start, or spread."""
+    small, t0 = _soup(seed, n, res, 0.5, 3)
+    big, t1 = _soup(seed + 1, wide, res, lo, hi, axis_scale)
+    tets = np.concatenate([t0, t1 + len(small)]).astype(np.int32)
+    if where == "start":
+        tets = np.roll(tets, wide, axis=0)
+    elif where == "spread":
+        tets = tets[np.random.default_rng(seed).permutation(len(tets))]
+    return np.concatenate([small, big]), np.ascontiguousarray(tets)
+
+
+@pytest.mark.parametrize("where", ["end", "start", "spread"])
+@pytest.mark.parametrize("n,wide,res,lo,hi", [(120000, 1, 64, 50, 64), (120000, 20, 64, 20, 64), (9000, 300, 64, 15, 40),
+                                              (9000, 65, 128, 60, 128), (300, 127, 128, 33, 100)])
+def test_wide_tets_among_small_ones(vt, n, wide, res, lo, hi, where):
+    """Only the tets with slices left go on to a tile's next window, shared by more threads: from one
+    tet of a tile to nearly all of them, several windows deep."""
+    verts, tets = _wide_among_small(n + wide, n, res, wide, lo, hi, where)
+    ref = oracle.voxelize(verts, tets, (0, 0, 0), 1.0 / res, res)
+    v, t = _cuda(verts, tets)
+    ws = vt.alloc_workspace(len(tets), len(verts), res)
+    got = vt.voxelize(v, t, (0, 0, 0), 1.0 / res, res, workspace=ws)
+    _same(got, ref, "one call")
+    flat = len(range(8, n, 17)) + len(range(8, wide, 17))
+    assert vt.read_stats(ws)["degenerate_tets"] >= flat  # each counted once, in its first window
+    _same(vt.voxelize(v, t, (0, 0, 0), 1.0 / res, res, row_cull=2, mode=0), ref, "all rows")
+    from paper_2106_01326_gb300 import batch
+
+    specs = [batch.JobSpec(batch.Mesh(v, t), res, vt.alloc_grid(res)) for _ in range(3)]
+    assert batch.voxelize_batched(specs) == [vt.OK] * 3
+    for sp in specs:
+        _same(sp.out, ref, "batch")
+
+
+@pytest.mark.parametrize("dims,scale,lo,hi", [((24, 2600, 40), (0.3, 1, 0.3), 300, 2600), ((24, 1500, 150), (0.2, 1, 1), 60, 1500),
+                                              ((600, 30, 300), (1, 0.2, 1), 40, 300)])
+@pytest.mark.parametrize("z", [None, (3, 8)])
+def test_tall_tets_among_small_ones(vt, dims, scale, lo, hi, z):
+    """Tets of more than 1024 rows, with and without more slices than a window holds, among small ones,
+    in whole grids and in slabs listed first."""
+    h = 1.0 / 4096
+    verts, tets = _wide_among_small(dims[1], 3000, max(dims), 30, lo, hi, "spread", scale)
+    verts = (verts * np.array([d * h for d in dims])).astype(np.float32)
+    z0, z1 = z or (0, dims[2])
+    ref = oracle.voxelize_grid(verts, tets, (0, 0, 0), h, dims, z0=z0, z1=z1)
+    v, t = _cuda(verts, tets)
+    for mode_cull in (0, 2):
+        _same(vt.voxelize_grid(v, t, (0, 0, 0), h, dims, z_range=(z0, z1), row_cull=mode_cull), ref, (dims, z, mode_cull))
