@@ -662,14 +662,14 @@ __global__ void __launch_bounds__(kListBlock) k_slab_list(Params p) {
   chain_wait();  // vertices snapped, header zeroed
   chain_release();
   __shared__ uint32_t warp_n[kListBlock / 32];
-  __shared__ float warp_rows[kListBlock / 32];
+  __shared__ unsigned warp_rows[kListBlock / 32], warp_slices[kListBlock / 32];
   __shared__ uint32_t first;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   TileCounters ctr;
   for (long long base = (long long)blockIdx.x * kListBlock; base < p.n_tets; base += (long long)gridDim.x * kListBlock) {
     const long long t = base + tid;
     bool keep = false;
-    unsigned rows = 0;
+    unsigned rows = 0, slices = 0;
     int3 V[4];
     if (t < p.n_tets && load_tet(p, t, V, ctr.err)) {
       Box bx;
@@ -680,30 +680,38 @@ __global__ void __launch_bounds__(kListBlock) k_slab_list(Params p) {
         const bool wide = E > kNarrowExtent;
         ctr.wide += wide;
         keep = !(wide || p.exact_all || bx.nb > kMaxFilterRows);
-        if (keep) rows = (unsigned)bx.nb * (unsigned)bx.nc;
-        else p.tetq[atomicAdd(&p.hdr->tetq_count, 1u)] = (uint32_t)t;
+        if (keep) {
+          rows = min((unsigned)bx.nb * (unsigned)bx.nc, 1u << 26);  // a warp's sum stays below 2^32
+          slices = (unsigned)bx.nc;
+        } else {
+          p.tetq[atomicAdd(&p.hdr->tetq_count, 1u)] = (uint32_t)t;
+        }
       }
     }
     const unsigned m = __ballot_sync(0xFFFFFFFFu, keep);
-    float r = (float)rows;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, d);
+    rows = __reduce_add_sync(0xFFFFFFFFu, rows);
+    slices = __reduce_add_sync(0xFFFFFFFFu, slices);
     if (lane == 0) {
       warp_n[warp] = __popc(m);
-      warp_rows[warp] = r;
+      warp_rows[warp] = rows;
+      warp_slices[warp] = slices;
     }
     __syncthreads();
     if (tid == 0) {
       uint32_t n = 0;
-      float all = 0.f;
-      for (int w = 0; w < kListBlock / 32; ++w) all += warp_rows[w];
+      unsigned long long all_rows = 0, all_slices = 0;
       for (int w = 0; w < kListBlock / 32; ++w) {
         const uint32_t c = warp_n[w];
         warp_n[w] = n;
         n += c;
+        all_rows += warp_rows[w];
+        all_slices += warp_slices[w];
       }
       first = n ? atomicAdd(&p.hdr->listq_count, n) : 0u;
-      if (n) atomicAdd(&p.hdr->list_rows, (unsigned long long)all);
+      if (n) {
+        atomicAdd(&p.hdr->list_rows, all_rows);
+        atomicAdd(&p.hdr->list_slices, all_slices);
+      }
     }
     __syncthreads();
     if (keep) p.tetq[p.n_tets - 1 - (long long)(first + warp_n[warp] + __popc(m & ((1u << lane) - 1u)))] = (uint32_t)t;

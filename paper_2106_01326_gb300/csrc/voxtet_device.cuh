@@ -49,8 +49,9 @@ struct Header {
   unsigned long long rows;
   unsigned long long degenerate;
   unsigned long long wide;
-  unsigned long long list_rows;  // rows of their boxes, over all slices
-  unsigned long long reserved[24];
+  unsigned long long list_rows;    // rows of their boxes, over all slices
+  unsigned long long list_slices;  // slices of their boxes
+  unsigned long long reserved[23];
 };
 static_assert(sizeof(Header) == 256, "header is 256 bytes");
 

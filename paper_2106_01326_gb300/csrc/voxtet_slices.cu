@@ -503,8 +503,10 @@ __global__ void __launch_bounds__(kSuBlock, SL == kSuSlicesSmall ? 7 : 5) k_slic
   unsigned rows = 0;
   const long long end = LIST ? (long long)p.hdr->listq_count : p.n_tets;
   int lg = p.lg;
-  if (LIST && end > 0) {  // as su_group_log2, with the slab's tets counted and their rows added up
+  if (LIST && end > 0) {  // as su_group_log2, with the slab's tets counted and their slices and rows added up
     const float slab = (float)(p.z1 - p.z0), per_tet = 0.5f * (float)p.hdr->list_rows / (float)end;
+    const float slices = (float)p.hdr->list_slices / (float)end;
+    while (lg < kSuMaxGroup && (float)(SL << lg) < slices) ++lg;
     while (lg < kSuMaxGroup && (float)(1 << lg) < slab &&
            (((end << lg) / kSuBlock) * 2 < (long long)gridDim.x ||
             su_share_more((end << lg) / kSuBlock, (long long)gridDim.x, per_tet, lg)))

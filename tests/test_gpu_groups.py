@@ -215,3 +215,15 @@ def test_tall_tets_among_small_ones(vt, dims, scale, lo, hi, z):
     v, t = _cuda(verts, tets)
     for mode_cull in (0, 2):
         _same(vt.voxelize_grid(v, t, (0, 0, 0), h, dims, z_range=(z0, z1), row_cull=mode_cull), ref, (dims, z, mode_cull))
+
+
+@pytest.mark.parametrize("z0,z1", [(300, 325), (400, 410)])
+def test_slab_of_long_thin_tets(vt, z0, z1):
+    """A slab's listed tets of 25 and 10 slices and a few rows each, shared by as many threads as hold
+    their slices in one window."""
+    dims, h = (30, 24, 900), 1.0 / 1024
+    verts, tets = _soup(77, 4000, 900, 20, 300, (0.01, 0.01, 1.0))
+    verts = (verts * np.array([d * h for d in dims])).astype(np.float32)
+    ref = oracle.voxelize_grid(verts, tets, (0, 0, 0), h, dims, z0=z0, z1=z1)
+    v, t = _cuda(verts, tets)
+    _same(vt.voxelize_grid(v, t, (0, 0, 0), h, dims, z_range=(z0, z1)), ref, (z0, z1))
