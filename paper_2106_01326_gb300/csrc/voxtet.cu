@@ -1224,7 +1224,8 @@ static int run_voxelize(const Workspace &w, long long n_verts, const int32_t *te
     p.exact_all = o.use_filter ? 0 : 1;
     const bool cull = o.row_cull == 1 || (o.row_cull == 0 && g.longest() >= kCullMinRes);
     const bool clamp = g.longest() >= kClampMinRes;
-    // Slabs thinner than an eighth of the grid take strided tiles (their tets are a thin band
+    // Slabs thinner than an eighth of the grid: slice units take a list of their tets (below), the span
+    // kernel strided tiles (their tets are a thin band
     // of a mesh numbered along z, which contiguous tiles would hand to a few blocks); thicker
     // slabs keep contiguous tiles, whose spatially coherent ORs use L2 better (measured on
     // GB300, brick-sparse torus: 4096^3 in quarter slabs 17.7 ms strided, 11.5 contiguous;
@@ -1250,7 +1251,12 @@ static int run_voxelize(const Workspace &w, long long n_verts, const int32_t *te
     if (grid > tiles) grid = tiles;
     if (o.profile && profile_begin(stream) != cudaSuccess) return VOXTET_ERR_CUDA;
     if (use_slice_units(o)) {
-      if (strided) {
+      // not for up to 4 slices of a mesh of up to 2^18 tets: few threads a tet can share such a slab, and
+      // tiles of all tets give a resident thread two or three (measured on GB300, list -> no list: 384 tets,
+      // 1 slice of 256^3 37.4 -> 31.2 us; 24,576 tets, 4 of 512^3 25.1 -> 22.9; 162,000 tets, 2 of 512^3
+      // 24.9 -> 20.4, but 8 slices 25.3 -> 35.6; 2.3 M tets, 1 slice 41.9 -> 46.3)
+      const bool list = strided && !(g.z1 - g.z0 <= 4 && n_tets <= (1 << 18));
+      if (list) {
         long long blocks = (n_tets + kListBlock - 1) / kListBlock;
         if (blocks > (long long)dev->sms * 8) blocks = (long long)dev->sms * 8;
         if (launch_chained(k_slab_list, (unsigned)blocks, kListBlock, 0, stream, p) != cudaSuccess)
@@ -1262,7 +1268,8 @@ static int run_voxelize(const Workspace &w, long long n_verts, const int32_t *te
       // (measured on GB300, sliver mesh 512^3: 308 -> 285 us with 16; a 4096^3 torus in slabs 4.19 ms
       // with 32, 4.28 with 16)
       const int cap = g.longest() <= 512 ? kSuSlicesSmall : kSuSlices;
-      if (launch_slices(p, variant >> 1, cap, dev->sms, stream) != VOXTET_OK) return VOXTET_ERR_CUDA;
+      const int sv = (list ? 4 : 0) | (o.mode == 1 ? 2 : 0) | (cull ? 1 : 0);
+      if (launch_slices(p, sv, cap, strided, dev->sms, stream) != VOXTET_OK) return VOXTET_ERR_CUDA;
       g_launches.fetch_add(1);
     } else {
       if (launch_chained(voxelize_kernel(variant), (unsigned)grid, kBlock, slice_table_bytes(p.max_slices), stream,
@@ -1686,10 +1693,10 @@ static size_t build_batch_image(const voxtet_job *jobs, int n, int cap, const vo
     if (ok[j] && !J.fixed_point) d.s = snap_args(J.origin, J.voxel_size, k);
     d.grid_words = ok[j] ? (long long)res * res * d.p.W : 0;
     d.clear = (ok[j] && !o.accumulate) ? 1 : 0;
+    d.p.tile_tets = kSuBlock >> d.p.lg;
     tiles[j] = tsum;
     pbase[j] = psum;
-    const int per_tile = kSuBlock >> d.p.lg;
-    tsum += (unsigned long long)((nt + per_tile - 1) / per_tile);
+    tsum += (unsigned long long)((nt + d.p.tile_tets - 1) / d.p.tile_tets);
     psum += prep_chunks(d);
   }
   tiles[n] = tsum;

@@ -82,6 +82,7 @@ struct Params {
   long long big_tiles;  // single-mesh launch: tiles of kTile tets before the kSmallTile tail
   long long tile_stride;  // > 0: tile k holds tets k + j * tile_stride (slab launches), else contiguous tiles
   int lg;           // slice-unit kernel: log2 of the threads that share a tet
+  int tile_tets;    // slice-unit kernel: tets per tile, at most 128 >> lg (0: chosen by the kernel, for lists)
   int vflags;       // exact kernel: 1 = fold the vertices' error bits (verts4[i].w) into the status
 };
 

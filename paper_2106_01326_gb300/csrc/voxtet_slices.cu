@@ -71,10 +71,10 @@ struct SuSmem {
   long long tile;
   int c0, r0;            // the current window: slices from c0, rows from r0 of each tet's box
   int next_c0, next_r0;  // the window after it (0, 0: the tile is done)
-  // the current window's tets, 2^lg threads each: all of the tile (n_sel = 0, lg = tile_lg) or the
+  // the current window's tets, 2^lg threads each: all tile_tets of the tile (n_sel = 0, lg = tile_lg) or the
   // n_sel at places place[buf] of it; those of the next window are collected in the other list.
   // (Read from here where they are used: held across the phases they cost the row loop registers.)
-  int lg, tile_lg, n_sel, n_next, buf;
+  int lg, tile_lg, tile_tets, n_sel, n_next, buf;
   uint8_t place[2][kSuBlock];
   // the block's counters but for the rows, since the last flush
   unsigned long long spans;
@@ -300,7 +300,7 @@ __device__ __forceinline__ int su_place(const SuSmem<SL> &sm, int slot) {
 // ... and in the launch.
 template <int SL>
 __device__ __forceinline__ long long su_launch_place(const SuSmem<SL> &sm, int slot) {
-  return sm.tile * (kSuBlock >> sm.tile_lg) + su_place(sm, slot);
+  return sm.tile * sm.tile_tets + su_place(sm, slot);
 }
 
 // Phase (3): rows b0 .. b0 + n - 1 of slice k of the tet in `slot`.
@@ -379,9 +379,9 @@ __device__ __forceinline__ bool su_pass(const Params &p, long long end, SuSmem<S
   bool more = false, tall = false;
   const int n_sel = sm.n_sel, lg = sm.lg;
   int g = tid >> lg;
-  const bool any = n_sel == 0 || g < n_sel;
+  const bool any = g < (n_sel ? n_sel : sm.tile_tets);
   if (n_sel && any) g = sm.place[sm.buf][g];
-  const long long t = any ? su_tet<LIST>(p, sm.tile * (kSuBlock >> (n_sel ? sm.tile_lg : lg)) + g, end) : -1;
+  const long long t = any ? su_tet<LIST>(p, sm.tile * sm.tile_tets + g, end) : -1;
   const int nc = su_setup<STRICT, CULL, TALL, SL>(p, t, sm, more, tall);
   bool again;
   {
@@ -446,13 +446,14 @@ __device__ __forceinline__ bool su_next_window(SuSmem<SL> &sm) {
 }
 
 template <int SL>
-__device__ __forceinline__ void su_begin(SuSmem<SL> &sm, int tile_lg) {
+__device__ __forceinline__ void su_begin(SuSmem<SL> &sm, int tile_lg, int tile_tets) {
   for (int i = threadIdx.x; i < kSuCounters; i += kSuBlock) sm.hist[i] = 0u;
   if (threadIdx.x == 0) {
     sm.stage.n = 0;
     sm.c0 = sm.r0 = sm.next_c0 = sm.next_r0 = 0;
     sm.n_sel = sm.n_next = sm.buf = 0;
     sm.lg = sm.tile_lg = tile_lg;
+    sm.tile_tets = tile_tets;
     sm.spans = 0;
     sm.degenerate = sm.wide = 0u;
     sm.err = 0;
@@ -492,6 +493,15 @@ static __host__ __device__ __forceinline__ bool su_share_more(long long tiles, l
   return tiles < 4 * blocks && 50.0f * (float)((2 << lg) - 1) < rows;
 }
 
+// Tets per tile where a slab of few slices leaves its tets to few threads each: as many as give each of
+// `blocks` blocks a tile, if that is fewer than a tile's threads have room for.  (Full tiles put a few
+// coarse tets, each with hundreds of rows of many words, on a few of the SMs: 384 tets in one slice of a
+// 2048^3 grid 191 -> 136 us, 3,072 in one of 512^3 28.7 -> 25.0; spans 159 and 26.9.)
+static __host__ __device__ __forceinline__ int su_tile_tets(long long tets, int lg, long long blocks) {
+  const long long room = kSuBlock >> lg, even = (tets + blocks - 1) / blocks;
+  return (int)(even < 1 ? 1 : even < room ? even : room);
+}
+
 // LIST: the tets are the hdr->listq_count ones listed at the back of p.tetq.  PAIRS: rows are ORed in
 // pairs of words.
 template <bool STRICT, bool CULL, bool PAIRS, bool LIST, int SL>
@@ -512,12 +522,12 @@ __global__ void __launch_bounds__(kSuBlock, SL == kSuSlicesSmall ? 7 : 5) k_slic
             su_share_more((end << lg) / kSuBlock, (long long)gridDim.x, per_tet, lg)))
       ++lg;
   }
-  su_begin(sm, lg);
+  su_begin(sm, lg, LIST ? su_tile_tets(end, lg, (long long)gridDim.x) : p.tile_tets);
   bool again = false;
   for (;;) {
     if (threadIdx.x == 0 && (!again || su_next_window(sm))) sm.tile = (long long)atomicAdd(&p.hdr->tile_counter, 1ull);
     __syncthreads();
-    if (sm.tile * (kSuBlock >> sm.tile_lg) >= end) break;
+    if (sm.tile * sm.tile_tets >= end) break;
     again = su_pass<STRICT, CULL, PAIRS, SL == kSuSlices, LIST, false, SL>(p, end, sm, rows);
   }
   su_flush(p.hdr, sm, rows);
@@ -540,7 +550,7 @@ __global__ void __launch_bounds__(kSuBlock, 7) k_slices_batched(BatchHeader *bh,
   __shared__ unsigned long long at, claim_end, job_first, job_end;
   const int tid = threadIdx.x;
   unsigned rows = 0;
-  su_begin(sm, 0);
+  su_begin(sm, 0, kSuBlock);
   const int n = bh->n_jobs;
   const unsigned long long total = bh->total_tiles, chunk = bh->chunk;
   int cur = -1;
@@ -583,7 +593,10 @@ __global__ void __launch_bounds__(kSuBlock, 7) k_slices_batched(BatchHeader *bh,
       __syncthreads();
       if (tid < (int)(sizeof(Params) / sizeof(uint32_t)))
         reinterpret_cast<uint32_t *>(&sp)[tid] = reinterpret_cast<const uint32_t *>(&jobs[j].p)[tid];
-      if (tid == 0) sm.lg = sm.tile_lg = jobs[j].p.lg;  // a new job's tile is at its first window
+      if (tid == 0) {  // a new job's tile is at its first window
+        sm.lg = sm.tile_lg = jobs[j].p.lg;
+        sm.tile_tets = jobs[j].p.tile_tets;
+      }
       __syncthreads();
       cur = j;
     }
@@ -671,7 +684,7 @@ int launch_slices_batched(BatchHeader *bh, const JobDesc *jobs, const unsigned l
   return e == cudaSuccess ? VOXTET_OK : VOXTET_ERR_CUDA;
 }
 
-int launch_slices(const Params &p_in, int variant, int slices, int sms, cudaStream_t stream) {
+int launch_slices(const Params &p_in, int variant, int slices, bool spread, int sms, cudaStream_t stream) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kSuMaxDevices) return VOXTET_ERR_CUDA;
   // Pairs of words where the ORs are the bound (32-slice windows: grids above 512 per side) and every
@@ -701,8 +714,8 @@ int launch_slices(const Params &p_in, int variant, int slices, int sms, cudaStre
   // a list's length is known on the device only: the kernel shares its tets among more threads
   const int side = 1 << (kLatticeBits - p.sh);
   p.lg = list ? 0 : su_group_log2(p.n_tets, side, p.ry, p.z1 - p.z0, slices, grid);
-  const int per_tile = kSuBlock >> p.lg;
-  const long long tiles = list ? grid : (p.n_tets + per_tile - 1) / per_tile;
+  p.tile_tets = spread ? su_tile_tets(p.n_tets, p.lg, grid) : kSuBlock >> p.lg;
+  const long long tiles = list ? grid : (p.n_tets + p.tile_tets - 1) / p.tile_tets;
   if (grid > tiles) grid = tiles;
   if (grid < 1) grid = 1;
   return launch_chained(kern, (unsigned)grid, kSuBlock, smem, stream, p) == cudaSuccess ? VOXTET_OK : VOXTET_ERR_CUDA;

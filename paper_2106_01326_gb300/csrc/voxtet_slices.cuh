@@ -31,8 +31,9 @@ int su_group_log2(long long n_tets, int side, int ry, int slab, int slices, long
 
 // Enqueue the slice-unit kernel for p on `stream`: variant = (list << 2) | (strict << 1) | cull;
 // slices = the slices a thread takes per window (kSuSlicesSmall or kSuSlices); list = the tets are
-// those k_slab_list listed.  Returns VOXTET_OK or VOXTET_ERR_CUDA.
-int launch_slices(const Params &p, int variant, int slices, int sms, cudaStream_t stream);
+// those k_slab_list listed; spread = over all resident blocks, if need be in tiles of fewer tets (lists
+// always are).  Returns VOXTET_OK or VOXTET_ERR_CUDA.
+int launch_slices(const Params &p, int variant, int slices, bool spread, int sms, cudaStream_t stream);
 
 // Enqueue the slice-unit kernel over a batch's jobs (tile_base: the jobs' tile offsets, tiles of
 // kSuBlock >> lg tets); its resident blocks per SM (0 on a CUDA error).

@@ -227,3 +227,21 @@ def test_slab_of_long_thin_tets(vt, z0, z1):
     ref = oracle.voxelize_grid(verts, tets, (0, 0, 0), h, dims, z0=z0, z1=z1)
     v, t = _cuda(verts, tets)
     _same(vt.voxelize_grid(v, t, (0, 0, 0), h, dims, z_range=(z0, z1)), ref, (z0, z1))
+
+
+@pytest.mark.parametrize("n,dims,lo,hi,scale", [(1, (40, 2100, 48), 30, 60, (0.3, 1, 1)), (5, (700, 300, 48), 10, 60, (1, 1, 1)),
+                                                (300, (64, 64, 64), 5, 60, (1, 1, 1)), (5000, (64, 64, 64), 1, 20, (1, 1, 1)),
+                                                (270000, (64, 64, 64), 0.3, 2, (1, 1, 1)), (40, (24, 20, 900), 30, 300, (0.1, 0.1, 1))])
+@pytest.mark.parametrize("nz", [1, 2, 4, 5, 7])
+def test_slabs_of_a_few_slices(vt, n, dims, lo, hi, scale, nz):
+    """Up to four slices of a small mesh go without a list, in tiles of fewer tets where those are few;
+    thicker slabs and larger meshes through a list."""
+    h = 1.0 / 4096
+    verts, tets = _soup(n, n, max(dims[2], 48), lo, hi, scale)
+    verts = (verts * np.array([d * h for d in dims])).astype(np.float32)
+    z0 = dims[2] // 2 - 1
+    ref = oracle.voxelize_grid(verts, tets, (0, 0, 0), h, dims, z0=z0, z1=z0 + nz)
+    v, t = _cuda(verts, tets)
+    for mode_cull in (0, 2):
+        got = vt.voxelize_grid(v, t, (0, 0, 0), h, dims, z_range=(z0, z0 + nz), row_cull=mode_cull)
+        _same(got, ref, (n, dims, nz, mode_cull))
