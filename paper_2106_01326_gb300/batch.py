@@ -80,6 +80,7 @@ def make_jobs(specs: Sequence[JobSpec]):
     one structured numpy array)."""
     pack = _ROW.pack
     rows = []
+    add = rows.append
     try:
         for sp in specs:
             mesh, origin = sp.mesh, sp.origin
@@ -87,8 +88,8 @@ def make_jobs(specs: Sequence[JobSpec]):
             if type(origin) is not tuple:  # numpy's rules: a single number, one for all three, [1, 3]
                 return _make_jobs_converting(specs)
             x, y, z = origin
-            rows.append(pack(v.data_ptr(), v.shape[0], t.data_ptr(), t.shape[0], x, y, z, sp.voxel_size, sp.res,
-                             sp.span_rows, 0, 0, sp.out.data_ptr()))
+            add(pack(v.data_ptr(), v.shape[0], t.data_ptr(), t.shape[0], x, y, z, sp.voxel_size, sp.res, sp.span_rows,
+                     0, 0, sp.out.data_ptr()))
     except (struct.error, OverflowError, TypeError, ValueError):
         return _make_jobs_converting(specs)
     return (vt.Job * max(len(rows), 1)).from_buffer(bytearray(b"".join(rows) or ctypes.sizeof(vt.Job)))

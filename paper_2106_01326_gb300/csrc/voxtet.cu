@@ -724,6 +724,11 @@ __global__ void __launch_bounds__(kListBlock) k_slab_list(Params p) {
 
 constexpr int kExactBlock = 128;
 constexpr int kExactBlocksPerSM = 7;  // 72 registers a thread
+// The batched form, whose Params come from the job table, would spill at 72 and is launched in fewer
+// blocks, each of which reads every job's counters: 256-job batch with few queued rows 13.1 us with 7
+// blocks per SM, 11.4 with 5; 64 jobs that queue most of their rows 2.02 and 2.25 ms (5.57 with 3 of 168
+// registers).
+constexpr int kExactBatchBlocksPerSM = 5;
 
 // A tet's exact face data in shared memory (Exact<i64> or Exact<i128>), faces in slot order.
 struct ExactTet {
@@ -956,8 +961,8 @@ __device__ __forceinline__ int queue_job(const u64 *pre, int m, u64 x) {
 // spread over all blocks: which jobs' rows need exact work is known only now (a job of wide tets on
 // a fine grid queues many times the rows of one with as many small tets).
 template <bool STRICT>
-__global__ void __launch_bounds__(kExactBlock, kExactBlocksPerSM) k_exact_batched(const BatchHeader *bh,
-                                                                                  const JobDesc *jobs) {
+__global__ void __launch_bounds__(kExactBlock, kExactBatchBlocksPerSM)
+    k_exact_batched(const BatchHeader *bh, const JobDesc *jobs) {
   __shared__ ExactTet sm;
   __shared__ u64 pre[kQueueJobs + 1];
   chain_wait();  // every row and tet is queued
@@ -1737,7 +1742,7 @@ static int launch_batch(char *ws, int cap, bool strict, bool cull, cudaStream_t 
   if (cudaGetLastError() != cudaSuccess) return VOXTET_ERR_CUDA;
   if (launch_slices_batched(bh, tab, tiles, status, strict, cull, dev->sms, stream) != VOXTET_OK) return VOXTET_ERR_CUDA;
   if (launch_chained(strict ? k_exact_batched<true> : k_exact_batched<false>,
-                     (unsigned)dev->sms * (unsigned)dev->occ_exact, kExactBlock, 0, stream, bh, tab) != cudaSuccess)
+                     (unsigned)dev->sms * kExactBatchBlocksPerSM, kExactBlock, 0, stream, bh, tab) != cudaSuccess)
     return VOXTET_ERR_CUDA;
   g_launches.fetch_add(kBatchLaunches);
   return VOXTET_OK;
