@@ -2112,12 +2112,13 @@ __global__ void __launch_bounds__(kCompactBlock) k_brick_count4(SlabBricks s, un
 }
 
 // One block: exclusive scan of the block counts in place, offset by the running total,
-// which then advances; the slab's device-detected status bits join the sticky bits.  Four counts a
+// which then advances; the slab's device-detected status bits join the sticky bits and, if another slab
+// follows, its header and redo bitmap are zeroed for it.  Four counts a
 // thread: a slab of the default size has 4096 blocks, one turn of the loop (a count a thread, four
 // turns: 6.6 us).
 __global__ void __launch_bounds__(1024) k_brick_scan(unsigned long long *counts, long long n_blocks,
                                                      SparseHeader *sh, Header *slab_hdr, uint32_t *redo,
-                                                     long long redo_words) {
+                                                     long long redo_words, unsigned q_cap) {
   __shared__ unsigned long long warp_sums[32];
   __shared__ unsigned long long carry;
   chain_wait();  // every brick is counted
@@ -2127,10 +2128,13 @@ __global__ void __launch_bounds__(1024) k_brick_scan(unsigned long long *counts,
     carry = sh->total;
     sh->sticky_bits |= slab_hdr->status_bits;
   }
+  const bool flagged = slab_hdr->rowq_count > q_cap;  // only then has any tet's bit been set
   __syncthreads();
   if (redo) {  // another slab follows: its launches find the header and the bitmap zeroed
     if (tid < (int)(sizeof(Header) / 4)) reinterpret_cast<uint32_t *>(slab_hdr)[tid] = 0u;
-    for (long long i = tid; i < redo_words; i += 1024) redo[i] = 0u;
+    // (the bitmap is one block's to clear: 83 us a slab for 35 M tets)
+    if (flagged)
+      for (long long i = tid; i < redo_words; i += 1024) redo[i] = 0u;
   }
   for (long long base = 0; base < n_blocks; base += 4096) {
     const long long i = base + 4 * tid;
@@ -2408,7 +2412,7 @@ int voxelize_tets_sparse(const float *d_verts, int64_t n_verts, const int32_t *d
     for (int sn = si + 1; sn < n_slabs; ++sn) last = last && !((marks[(size_t)sn >> 5] >> (sn & 31)) & 1u);
     if (e == cudaSuccess)
       e = launch_chained(k_brick_scan, 1u, 1024u, 0, stream, block_counts, nb, sh, w.hdr, last ? nullptr : w.redo,
-                         w.redo_words);
+                         w.redo_words, w.q_cap);
     if (e == cudaSuccess)
       e = launch_chained(k_brick_write, (unsigned)nb, kCompactBlock, 0, stream, s, block_counts, masks, d_brick_keys,
                          d_brick_words, (long long)max_bricks);

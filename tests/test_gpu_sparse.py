@@ -181,3 +181,17 @@ def test_sparse_dirty_scratch_and_reuse(vt):
         keys, words = vt.voxelize_sparse(dv, dt, (0, 0, 0), h, res3, slab_depth=depth, scratch=scratch)
         assert (keys.cpu().numpy().view(np.uint64) == rk).all()
         assert (words.cpu().numpy().view(np.uint32) == rw).all()
+
+
+@pytest.mark.parametrize("depth", [32, 64, 96])
+def test_sparse_row_queue_overflow(vt, depth):
+    """Cells of 4:12:12 voxels' thirds: about 1,850 uncertain rows a slice, so that slabs of 64 and 96
+    slices overflow the row queue (65,536) and flag tets, and the slab after them, of 64 or 32 slices,
+    starts from a cleared bitmap; slabs of 32 do not overflow it."""
+    res, n = 128, 12
+    ijk, t = mg.kuhn_lattice_int(n)
+    unit = (1 << 20) // (12 * n) // 2048 * 2048
+    xyz = ijk * (np.array([4, 12, 12]) * unit) + (1 << 19) // res
+    v = (xyz / (1 << 20)).astype(np.float32)
+    assert (v.astype(np.float64) * (1 << 20) == xyz).all()
+    _check(vt, v, t.astype(np.int32), 1.0 / res, (res, res, res), slab_depth=depth)
