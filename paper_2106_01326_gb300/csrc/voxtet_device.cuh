@@ -1,11 +1,10 @@
 // voxtet_device.cuh -- device-side types and helpers shared by the voxelizer's kernels.
 //
-// The workspace header, the per-launch parameters, the OR writes into the bit grid,
-// the checked tet load, the per-slice candidate-row range (edge lines of the tet's
-// cross-section), the exact row narrowing of faces parallel to x, the block-staged
-// queue of rows the filter could not certify and the per-block counters.  Both the
-// span kernel (voxtet.cu) and the slice-unit kernel (voxtet_slices.cu) use them, so
-// their grids and queues agree by construction.
+// Used by the span kernel (voxtet.cu) and the slice-unit kernel (voxtet_slices.cu) alike: the
+// workspace header, the per-launch parameters, the checked tet load, the exact row narrowing of faces
+// parallel to x and the block-staged queue of rows the filter could not certify.  The span kernel's
+// own: the OR of a row and the candidate rows of a slice from the edges of its cross-section (the
+// slice-unit kernel's are in voxtet_rows.cuh).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>

@@ -20,12 +20,13 @@
 // past that are taken in further windows of the same tile, by the tets that have them.  A batch's jobs run in one launch
 // (k_slices_batched), a thin slab's tets from a list (LIST).
 // What bounds it: instruction issue and, on finer grids, the rate at which ORs reach L2, half of
-// them across the dies.  Measured on GB300 with timing-only copies, 1.3 M-tet sliver mesh: at
-// 512^3 261 us a call, of these 65 for the ORs, 100 for the rest of the rows, 45 for the slices'
-// row ranges and the sort, 40 for load, classification and face data; at 1024^3 1020 us, 505 for
-// the ORs (213 M of them) and 360 for the rest of the rows.  ORing a tile's rows in shared memory
-// first and the words once into the grid took 9 times fewer ORs but a sixth more instructions
-// (302 and 1100 us).
+// them across the dies.  Measured on GB300, 1.3 M-tet sliver mesh: 257 us a call at 512^3, 990 at
+// 1024^3 (rows ORed in pairs of words).  Timing-only copies of a form that ORed single words at both
+// sizes: at 512^3 261 us a call, of these 65 for the ORs, 100 for the rest of the rows, 45 for the
+// slices' row ranges and the sort, 40 for load, classification and face data; at 1024^3 1020 us, 505
+// for the ORs (213 M of them) and 360 for the rest of the rows.  ORing a tile's rows in shared memory
+// first and the words once into the grid took 9 times fewer ORs but a sixth more instructions (302 and
+// 1100 us).
 // Tets wider than 2^20 lattice units (or all, use_filter = 0) go to the exact kernel, zero-volume
 // ones are counted; rows the filter cannot certify go to the row queue, as in the span kernel.
 #include <cuda_runtime.h>
@@ -690,7 +691,9 @@ int launch_slices(const Params &p_in, int variant, int slices, bool spread, int 
   // Pairs of words where the ORs are the bound (32-slice windows: grids above 512 per side) and every
   // row starts on an 8-byte boundary.  Measured on GB300: sliver mesh at 1024^3 1018 -> 996 us,
   // 162,000 tets at 1024^3 656 -> 606, 1.3 M at 2048^3 4.77 -> 4.40 ms, 4096^3 torus in slabs 4.22 ->
-  // 3.89 ms; at 512^3, bound by issue, the longer masks cost more than they save.
+  // 3.89 ms; at 512^3, bound by issue, the longer masks cost more than they save.  They also do where a
+  // mesh on a lattice puts the same rows of many tets side by side: 1.3 M tets of 6 x 9 x 15 voxels at
+  // 1024^3 543 -> 577 us, of 17 x 17 x 17 839 -> 981.
   const int c = slices <= kSuSlicesSmall ? 0 : (p_in.W & 1) != 0 || (reinterpret_cast<uintptr_t>(p_in.out) & 7) != 0 ? 1 : 2;
   const SuKernel kern = c == 0   ? su_kernel<false, kSuSlicesSmall>(variant & 7)
                         : c == 1 ? su_kernel<false, kSuSlices>(variant & 7)
